@@ -62,7 +62,8 @@ L2_FLUSH_BYTES = 256 << 20
 # traffic is per event: momenta in, |M|^2 out).  Reported as null once the
 # sources differ from the captured ones (kernel_digest()).
 NCU_TRAFFIC = {"ggttgg": (65536, 12815104 + 745216, "bd63ce2f23a8d439")}
-KERNEL_SOURCES = ("mg_kernels.cuh", "mg_vertices.cuh", "mg_colour_tc.cuh", "mg_flowstore.cuh")
+KERNEL_SOURCES = ("mg_kernels.cuh", "mg_vertices.cuh", "mg_colour_tc.cuh", "mg_recursion.cuh",
+                  "mg_recursion_kernels.cuh")
 
 SERVE_PROCS = {  # process -> sqrt(s)
     "e+ e- > mu+ mu-": 500.0,
@@ -171,13 +172,28 @@ def load_flops(tag: str) -> dict:
 def launches_per_sigma(proc: str, nevt: int, ngood: int) -> int:
     """Kernel launches of one mixed mg_sigma call: one, except for gg -> t t~ g g g,
     whose two-phase path launches the flow and colour kernels once per slice
-    of the good helicities, the slices sized to a 1 GiB flow workspace
-    (120 complex FP32 flows per helicity-event row, events padded to 128)."""
+    of the events, the slices sized to the workspace (at most 1 GiB: as many
+    rows of 120 complex FP32 flows of one helicity over the events, padded to
+    128, as fit, shared out as 128 helicities per event)."""
     if proc != "ggttggg":
         return 1
     per_hel = 120 * ((nevt + 127) // 128 * 128) * 8
     hs = max(1, min(ngood, (1 << 30) // per_hel))
-    return 2 * ((ngood + hs - 1) // hs)
+    slice_events = hs * per_hel // (120 * 128 * 8)
+    return 2 * ((nevt + slice_events - 1) // slice_events)
+
+
+def flops_per_event(fl: dict, ngood: int, recursion: bool) -> float:
+    """Algorithmic flops of one event: the helicity-shared recursion (all
+    helicities, counted with its colour form), or the per-helicity program."""
+    if recursion:
+        return fl["rec_flops_per_event"] + fl["rec_colour_flops_per_event"]
+    return ngood * (fl["amp_flops_per_hel"] + fl["colour_dense_flops_per_hel"])
+
+
+def uses_recursion(tag: str, prec: str) -> bool:
+    from paper_2303_18244_gb300.generator.emit import RECURSION
+    return tag in RECURSION[prec]
 
 
 def time_oracle(proc: str, sqrts: float, seed: int, first_event: int, budget_s: float = 12.0,
@@ -406,12 +422,13 @@ def main():
     uwb_bytes = 16 * 128 * nevt + 8 * uwb_kept
 
     fl = load_flops(args.proc)
-    flops_evt = ngood * (fl["amp_flops_per_hel"] + fl["colour_dense_flops_per_hel"])
+    flops_evt = flops_per_event(fl, ngood, uses_recursion(args.proc, "f32"))
+    flops_evt64 = flops_per_event(fl, ngood, uses_recursion(args.proc, "f64"))
     kernel_ms = t_mix / args.steps
     achieved = flops_evt * nevt / (kernel_ms * 1e-3) / 1e12
     peak32 = mg.diag_fma_peak(0) / 1e3
     peak64 = mg.diag_fma_peak(1) / 1e3
-    achieved64 = flops_evt * nevt / (t_64 * 1e-3) / 1e12
+    achieved64 = flops_evt64 * nevt / (t_64 * 1e-3) / 1e12
 
     traffic = traffic_per_launch(args.proc, nevt)
 
@@ -520,7 +537,7 @@ def measure_config(tag, mg, process_momenta, timed_call, peak32, peak64, oracle_
         ms = timed_call(lambda: mg.sigma(h, mom, out), 3, warm)
         assert mg.process_status(h) == 0
         t = statistics.median(ms)
-        flops = ngood * (fl["amp_flops_per_hel"] + fl["colour_dense_flops_per_hel"]) * nevt
+        flops = flops_per_event(fl, ngood, uses_recursion(tag, "f32" if name == "mixed" else "f64")) * nevt
         peak = peak32 if name == "mixed" else peak64
         r = {"value": nevt / (t * 1e-3), "unit": "MEs/s", "ms_per_step": t, "steps": len(ms),
              "good_helicities": ngood,
@@ -567,19 +584,19 @@ def two_phase_rooflines(h, mom, out, mg, fl, ngood, nevt):
     t1 = statistics.median(r[0] for r in runs)
     t2 = statistics.median(r[1] for r in runs)
     slices = runs[0][2]
-    rows = ngood * ((nevt + 127) // 128 * 128)
+    rows = 128 * nevt
     peak32 = mg.diag_fma_peak(0) / 1e3
     hbm = measured_peak("hbm_gbs")
     bf16 = measured_peak("bf16_tflops")
     fp16_mma = mg.diag_mma_peak()
-    f1 = ngood * fl["amp_flops_per_hel"] * nevt / (t1 * 1e-3) / 1e12
+    f1 = fl["rec_flops_per_event"] * nevt / (t1 * 1e-3) / 1e12
     b2 = rows * 120 * 8 / (t2 * 1e-3) / 1e9
-    f2 = 4 * 120 ** 2 * ngood * nevt / (t2 * 1e-3) / 1e12
+    f2 = 4 * 120 ** 2 * rows / (t2 * 1e-3) / 1e12
     return {
         "slices": slices,
-        "flows_tmem_kernel": {"ms": t1, "bound": "alu", "achieved": f1, "peak": peak32, "unit": "TFLOP/s",
+        "rec_flows_kernel": {"ms": t1, "bound": "alu", "achieved": f1, "peak": peak32, "unit": "TFLOP/s",
                               "frac": f1 / peak32, "peak_source": "measured FP32 FMA loop (mg_diag)"},
-        "colour_rows_tc_kernel": {"ms": t2, "bound": "hbm", "achieved": b2, "peak": hbm, "unit": "GB/s",
+        "rec_colour_tc_kernel": {"ms": t2, "bound": "hbm", "achieved": b2, "peak": hbm, "unit": "GB/s",
                                   "frac": b2 / hbm if hbm else None,
                                   "bytes_per_row": "960 (120 complex FP32 flows read once)",
                                   "peak_source": "measured copy bandwidth (hbm_gbs)",

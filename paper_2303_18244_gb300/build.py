@@ -53,7 +53,8 @@ def processes() -> list[str]:
 def generate() -> list[str]:
     """Write csrc/gen/<tag>.cuh, <tag>_f64.cu, <tag>_f32.cu and registry.cu; return the TUs."""
     sys.path.insert(0, ROOT)
-    from paper_2303_18244_gb300.generator.emit import PROCESSES, emit, emit_tu, header_name
+    from paper_2303_18244_gb300.generator.emit import PROCESSES, RECURSION, emit, emit_tu, header_name
+    from paper_2303_18244_gb300.generator.recursion import emit_recursion
     os.makedirs(GEN, exist_ok=True)
     tus = []
     procs = processes()
@@ -72,6 +73,9 @@ def generate() -> list[str]:
             if prec == "f64" or name != header_name(proc, "f64"):
                 tag, hdr = emit(proc, prec)
                 _write_if_changed(os.path.join(GEN, name), hdr)
+        tag, n = PROCESSES[proc]
+        if tag in RECURSION["f64"] | RECURSION["f32"]:
+            _write_if_changed(os.path.join(GEN, f"{tag}_rec.cuh"), emit_recursion(n, tag))
         for prec in ("f64", "f32"):
             _, tu = emit_tu(proc, prec)
             path = os.path.join(GEN, f"{tag}_{prec}.cu")

@@ -24,7 +24,6 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
-#include "mg_flowstore.cuh"
 #include "mg_kernels.cuh"
 
 namespace mg {
@@ -102,39 +101,6 @@ __host__ __device__ constexpr uint32_t tile_off(int row, int k, int K) {
 }
 
 }  // namespace tc
-
-// Shared-memory layout of the tensor-core kernel.  The momenta tile is dead
-// once the per-event set-up has run, so the operand tiles reuse its space.
-// With MG_TC_ALIAS the colour-flow accumulators share that space too (each
-// thread moves its flows into registers before the operand tiles are
-// written), which leaves the constant B tile and the slab as the only other
-// regions.
-#ifndef MG_TC_ALIAS
-#define MG_TC_ALIAS 0
-#endif
-template <class P, int NT>
-struct LayoutTC {
-  static constexpr bool alias = MG_TC_ALIAS != 0;
-  static constexpr int K = tc::pad16(P::NCOL);
-  static constexpr int N = tc::pad16(P::NCOL);
-  static constexpr size_t r128(size_t b) { return ((b + 127) / 128) * 128; }
-  static constexpr size_t a_tile = size_t(NT) * K * 2;  // FP16 [NT][K]
-  static constexpr size_t b_tile = size_t(N) * K * 2;   // FP16 [N][K]
-  static constexpr size_t bar_bytes = 128;               // TMA bar, MMA bar, TMEM address
-  static constexpr size_t stage_bytes = size_t(NT) * P::NPAR * 4 * sizeof(double);
-  static constexpr size_t jamp_bytes = size_t(NT) * P::NCOL * sizeof(cx<float>);
-  static constexpr size_t slab_bytes = size_t(NT) * slab_slots<P, float>() * sizeof(float);
-  static constexpr size_t ops_bytes = 4 * a_tile + (alias ? 0 : b_tile);
-  static constexpr size_t region_bytes = stage_bytes > ops_bytes
-                                             ? (alias && jamp_bytes > stage_bytes ? jamp_bytes : stage_bytes)
-                                             : (alias && jamp_bytes > ops_bytes ? jamp_bytes : ops_bytes);
-  static constexpr size_t region_off = bar_bytes;  // no-swizzle tiles need 16-byte alignment only
-  static constexpr size_t b_off = alias ? region_off + r128(region_bytes) : region_off + 4 * a_tile;
-  static constexpr size_t slab_off = alias ? b_off + r128(b_tile) : region_off + r128(region_bytes);
-  static constexpr size_t jamp_off = alias ? region_off : slab_off + r128(slab_bytes);
-  static constexpr size_t base_bytes = alias ? slab_off + r128(slab_bytes) : jamp_off + r128(jamp_bytes);
-  static constexpr uint32_t tmem_cols = (2 * N <= 32) ? 32 : (2 * N <= 64) ? 64 : (2 * N <= 128) ? 128 : 256;
-};
 
 // The per-helicity colour form of a CTA of 128 events, shared by the fused
 // kernels.  (1) Each event's thread writes its flows, scaled by a power of two
@@ -215,109 +181,6 @@ __device__ __forceinline__ float colour_readback(uint32_t lane_base, const float
   return dsum;
 }
 
-// CTAs per SM the register allocation is sized for (launch bounds).  At 2 the
-// straight-line gg -> t t~ g g code keeps 255 registers; 3 caps them at 168 and
-// its spills halve the throughput (measured).
-#ifndef MG_TC_MINB
-#define MG_TC_MINB 1
-#endif
-
-// Mixed-precision |M|^2 with the tensor-core colour sum; NT = 128 events per CTA.
-template <class P, int NT>
-__global__ void __launch_bounds__(NT, MG_TC_MINB) sigma_tc_kernel(const double* __restrict__ mom, long long nevt,
-                                                      double* __restrict__ me, const int* __restrict__ hels,
-                                                      int nhel, KParams kp, const uint4* __restrict__ ctile,
-                                                      unsigned* __restrict__ status) {
-  static_assert(NT == 128, "one event per TMEM lane");
-  using LY = LayoutTC<P, NT>;
-  constexpr int K = LY::K, N = LY::N;
-  extern __shared__ __align__(128) unsigned char smem[];
-  uint64_t* tma_bar = reinterpret_cast<uint64_t*>(smem);
-  uint64_t* mma_bar = reinterpret_cast<uint64_t*>(smem + 16);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 32);
-  unsigned char* region = smem + LY::region_off;
-  float* slab = reinterpret_cast<float*>(smem + LY::slab_off);
-  cx<float>* jamp = reinterpret_cast<cx<float>*>(smem + LY::jamp_off) + threadIdx.x;
-  const int tid = threadIdx.x;
-  const int warp = tid >> 5;
-
-  const int nvalid =
-      load_and_prepare_at<P, float, NT>(tma_bar, reinterpret_cast<double*>(region), slab, mom, nevt, kp, status);
-  if (nvalid < 0) return;  // (load_and_prepare_at ends with a block barrier: the tile space is free)
-
-  // colour matrix tile (constant), operand tiles, accumulators
-  unsigned char* atile = region;                    // 4 tiles: re_hi, re_lo, im_hi, im_lo
-  unsigned char* btile = smem + LY::b_off;
-  for (int i = tid; i < (int)(LY::b_tile / 16); i += NT)
-    reinterpret_cast<uint4*>(btile)[i] = __ldg(ctile + i);
-  if (tid == 0) {
-    mbar_init(mma_bar, 1);
-    fence_mbar_init();
-  }
-  if (warp == 0) {
-    tc::tmem_alloc(tmem_slot, LY::tmem_cols);
-    tc::tmem_relinquish();
-  }
-  fence_proxy_async_smem();
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
-  const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
-  const uint32_t a_addr = smem_u32(atile);
-  const uint32_t b_addr = smem_u32(btile);
-
-  double acc = 0.0;
-  uint32_t phase = 0;
-  bool ok = true;
-#pragma unroll 1
-  for (int ih = 0; ih < nhel && ok; ih++) {
-    const int h = __ldg(hels + ih);
-    P::template amplitudes<float>(slab + tid, NT, h, kp.v, jamp, NT);
-    // the event's flows into registers (their space may hold the operand tiles)
-    float fr[P::NCOL], fi[P::NCOL];
-#pragma unroll
-    for (int k = 0; k < P::NCOL; k++) {
-      fr[k] = jamp[k * NT].re;
-      fi[k] = jamp[k * NT].im;
-    }
-    if constexpr (LY::alias) __syncthreads();
-    // per-event power-of-two scale, FP16 hi/lo split into the operand tiles
-    const float s = colour_operands<P, K>(atile, LY::a_tile, tid, fr, fi);
-    fence_proxy_async_smem();  // generic-proxy tile writes -> visible to the tensor core
-    __syncthreads();
-    if (tid == 0) colour_mma<K, N>(tmem, a_addr, b_addr, LY::a_tile, mma_bar);
-    // the outcome of the bounded wait is made uniform across the CTA, so that
-    // no thread can skip the warp-collective TMEM loads or a barrier alone
-    if (!__syncthreads_and(mbar_wait_bounded(mma_bar, phase, kp.polls) ? 1 : 0)) {
-      if (tid == 0) atomicOr(status, ST_MMA_TIMEOUT);
-      ok = false;
-      break;
-    }
-    phase ^= 1u;
-    tc::fence_after_sync();
-    const float dsum = colour_readback<P, N>(lane_base, fr, fi);
-    acc += (double)(dsum / s);
-    tc::fence_before_sync();
-    __syncthreads();  // tiles and accumulators are reused by the next helicity
-  }
-  if (!ok) {
-    // an MMA did not signal completion: wait once more (bounded) before the
-    // accumulators are released, leave the outputs unwritten
-    mbar_wait_bounded(mma_bar, phase, WAIT_POLLS);
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) {
-    tc::fence_after_sync();
-    tc::tmem_dealloc(tmem, LY::tmem_cols);
-  }
-  if (ok && tid < nvalid) {
-    constexpr double norm = 1.0 / (P::IDEN * P::CDEN);
-    me[(long long)blockIdx.x * NT + tid] = acc * norm;
-  }
-}
-
 // FP16 bit pattern of an integer, or -1 if it is not exactly representable.
 inline int fp16_bits_of_int(int v) {
   if (v == 0) return 0;
@@ -346,18 +209,10 @@ inline bool colour_tile_host(const int* knum, int ncol, unsigned short* out /* [
 
 // ---------------------------------------------------------------------------
 // Two-phase mixed path for processes whose colour operands do not fit in
-// shared memory beside the per-event state (120 flows): flows_kernel writes
-// the FP32 flows of every (good helicity, event) row to a workspace in HBM;
-// colour_rows_tc_kernel contracts them with the colour matrix on the tensor
-// cores, batched over events x helicities, and sums the helicities per event.
+// shared memory beside the per-event state (120 flows): the FP32 flows of
+// every (event, helicity) row go to a workspace in HBM; a second kernel
+// contracts them with the colour matrix (mg_recursion_kernels.cuh).
 // ---------------------------------------------------------------------------
-// MG_ROWS_REGS (default 1): the colour kernel holds each row's flows in
-// registers for the helicity (see colour_rows_tc_kernel); 0 reads them from
-// the workspace where they are used.
-#ifndef MG_ROWS_REGS
-#define MG_ROWS_REGS 1
-#endif
-constexpr int ROWS_REGS = MG_ROWS_REGS;  // for the unroll counts (pragmas see no macros)
 template <class P>
 struct LayoutRows {
   static constexpr int K = tc::pad16(P::NCOL);
@@ -370,369 +225,12 @@ struct LayoutRows {
   static constexpr uint32_t tmem_cols = (2 * N <= 32) ? 32 : (2 * N <= 64) ? 64 : (2 * N <= 128) ? 128 : 256;
 };
 
-// One CTA per 128 rows of events (TMEM lane = event).  Per helicity of the
-// slice: the rows' flows from J (rows past nevt read as zero), a per-row
-// power-of-two scale, FP16 hi/lo operand tiles, D = A K in TMEM for Re and
-// Im, then sum_k J_k D_k with the FP32 flows; helicities summed in FP64 into
-// me: a later slice continues the running sum stored by the one before, so
-// the helicities are added in the same order however they are sliced; the
-// last slice normalises.
-template <class P>
-__global__ void __launch_bounds__(128, 1)
-    colour_rows_tc_kernel(const float2* __restrict__ J, long long ldj, long long nevt, double* __restrict__ me,
-                          int nhel, int first, int last, const uint4* __restrict__ ctile,
-                          unsigned* __restrict__ status, uint32_t polls) {
-  using LY = LayoutRows<P>;
-  constexpr int NT = 128, K = LY::K, N = LY::N;
-  static_assert(2 * N <= 256, "two accumulators of N columns");
-  extern __shared__ __align__(128) unsigned char smem[];
-  uint64_t* mma_bar = reinterpret_cast<uint64_t*>(smem);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 16);
-  unsigned char* atile = smem + LY::a_off;
-  unsigned char* btile = smem + LY::b_off;
-  const int tid = threadIdx.x;
-  const int warp = tid >> 5;
-  const long long e = (long long)blockIdx.x * NT + tid;
-  const bool valid = e < nevt;
-
-  for (int i = tid; i < (int)(LY::b_tile / 16); i += NT) reinterpret_cast<uint4*>(btile)[i] = __ldg(ctile + i);
-  if (tid == 0) {
-    mbar_init(mma_bar, 1);
-    fence_mbar_init();
-  }
-  if (warp == 0) {
-    tc::tmem_alloc(tmem_slot, LY::tmem_cols);
-    tc::tmem_relinquish();
-  }
-  fence_proxy_async_smem();
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
-  const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
-  constexpr uint32_t idesc = tc::idesc_f16(128, N);
-  const uint32_t a_addr = smem_u32(atile);
-  const uint32_t b_addr = smem_u32(btile);
-  constexpr uint32_t SBO = (K / 8) * 128;
-
-  double acc = (!first && valid) ? me[e] : 0.0;
-  uint32_t phase = 0;
-  bool ok = true;
-#pragma unroll 1
-  for (int ih = 0; ih < nhel && ok; ih++) {
-    const float2* row = J + (long long)ih * P::NCOL * ldj + e;
-#if MG_ROWS_REGS
-    // the row's flows into registers with every load in flight at once (one
-    // read of the workspace; the loads of a loop that used each value at
-    // once kept only a few per thread in flight)
-    float2 fv[P::NCOL];
-#pragma unroll
-    for (int k = 0; k < P::NCOL; k++) fv[k] = valid ? __ldcs(row + (long long)k * ldj) : make_float2(0.f, 0.f);
-#define MG_ROW_FLOW(k) fv[k]
-#else
-#define MG_ROW_FLOW(k) row[(long long)(k) * ldj]
-#endif
-    float mx = 0.f;
-    if (valid) {
-#pragma unroll ROWS_REGS ? P::NCOL : 8
-      for (int k = 0; k < P::NCOL; k++) {
-        const float2 v = MG_ROW_FLOW(k);
-        mx = fmaxf(mx, fmaxf(fabsf(v.x), fabsf(v.y)));
-      }
-    }
-    const int ex = mx > 0.f ? ((int)((__float_as_uint(mx) >> 23) & 0xff) - 127) : 0;
-    const float s = __uint_as_float((uint32_t)(127 - ex) << 23);  // 2^-ex
-#pragma unroll ROWS_REGS ? K / 8 : 1
-    for (int j = 0; j < K / 8; j++) {
-      __align__(16) __half hr[8], lr[8], hi_[8], li[8];
-#pragma unroll
-      for (int q = 0; q < 8; q++) {
-        const int k = 8 * j + q;
-        const float2 v = (valid && k < P::NCOL) ? MG_ROW_FLOW(k < P::NCOL ? k : 0) : make_float2(0.f, 0.f);
-        const float xr = s * v.x, xi = s * v.y;
-        hr[q] = __float2half_rn(xr);
-        lr[q] = __float2half_rn(xr - __half2float(hr[q]));
-        hi_[q] = __float2half_rn(xi);
-        li[q] = __float2half_rn(xi - __half2float(hi_[q]));
-      }
-      const uint32_t off = tc::tile_off(tid, 8 * j, K);
-      *reinterpret_cast<uint4*>(atile + 0 * LY::a_tile + off) = *reinterpret_cast<const uint4*>(hr);
-      *reinterpret_cast<uint4*>(atile + 1 * LY::a_tile + off) = *reinterpret_cast<const uint4*>(lr);
-      *reinterpret_cast<uint4*>(atile + 2 * LY::a_tile + off) = *reinterpret_cast<const uint4*>(hi_);
-      *reinterpret_cast<uint4*>(atile + 3 * LY::a_tile + off) = *reinterpret_cast<const uint4*>(li);
-    }
-    fence_proxy_async_smem();  // generic-proxy tile writes -> visible to the tensor core
-    __syncthreads();
-    if (tid == 0) {
-      tc::fence_after_sync();
-      for (int part = 0; part < 2; part++) {  // 0: Re -> columns [0, N), 1: Im -> [N, 2N)
-        const uint32_t d = tmem + part * N;
-        for (int kk = 0; kk < K / 16; kk++) {
-          const uint64_t bd = tc::smem_desc(b_addr + kk * 2 * tc::LBO, tc::LBO, SBO);
-          const uint32_t hi_base = a_addr + (2 * part) * (uint32_t)LY::a_tile + kk * 2 * tc::LBO;
-          const uint32_t lo_base = a_addr + (2 * part + 1) * (uint32_t)LY::a_tile + kk * 2 * tc::LBO;
-          tc::mma_f16(d, tc::smem_desc(hi_base, tc::LBO, SBO), bd, idesc, kk > 0 ? 1u : 0u);
-          tc::mma_f16(d, tc::smem_desc(lo_base, tc::LBO, SBO), bd, idesc, 1u);
-        }
-      }
-      tc::mma_commit(mma_bar);
-    }
-    // bounded wait, outcome uniform across the CTA (see sigma_tc_kernel)
-    if (!__syncthreads_and(mbar_wait_bounded(mma_bar, phase, polls) ? 1 : 0)) {
-      if (tid == 0) atomicOr(status, ST_MMA_TIMEOUT);
-      ok = false;
-      break;
-    }
-    phase ^= 1u;
-    tc::fence_after_sync();
-    float dsum = 0.f;
-#pragma unroll ROWS_REGS ? N / 16 : 1
-    for (int c = 0; c < N; c += 16) {
-      float dr[16], di[16];
-      tc::tmem_ld16(lane_base + c, dr);
-      tc::tmem_ld16(lane_base + N + c, di);
-      tc::tmem_wait_ld();
-#pragma unroll
-      for (int q = 0; q < 16; q++) {
-        const int k = c + q;
-        const float2 v = (valid && k < P::NCOL) ? MG_ROW_FLOW(k < P::NCOL ? k : 0) : make_float2(0.f, 0.f);
-        dsum = fmaf(v.x, dr[q], dsum);
-        dsum = fmaf(v.y, di[q], dsum);
-      }
-    }
-#undef MG_ROW_FLOW
-    acc += (double)(dsum / s);
-    tc::fence_before_sync();
-    __syncthreads();  // tiles and accumulators are reused by the next helicity
-  }
-  if (!ok) mbar_wait_bounded(mma_bar, phase, WAIT_POLLS);
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) {
-    tc::fence_after_sync();
-    tc::tmem_dealloc(tmem, LY::tmem_cols);
-  }
-  if (ok && valid) {
-    constexpr double norm = 1.0 / (P::IDEN * P::CDEN);
-    me[e] = last ? acc * norm : acc;
-  }
-}
-
-// First phase with the colour flows in tensor memory (default; MG_FLOWS_TMEM=0
-// selects flows_kernel): 128 events per CTA, TMEM lane = event, two columns
-// per flow; shared memory holds only the momenta tile and the per-event slab,
-// so that two CTAs (8 warps) fit on an SM instead of two CTAs of 64 events.
-// Same output as flows_kernel; gg -> t t~ g g g mixed 1.79e5 -> 2.87e5 MEs/s.
-#ifndef MG_FLOWS_TMEM
-#define MG_FLOWS_TMEM 1
-#endif
-// MG_FLOWS_NT: events per CTA of the tensor-memory flow kernel, 128 (two
-// CTAs of 4 warps per SM) or 256 (one CTA of 8 warps per SM holding all 512
-// TMEM columns: warp w keeps its 32 events in lanes 32 (w mod 4) and the
-// column half w / 4, so that with MG_CHUNK_SYNC all 8 warps of an SM run the
-// same chunk of the helicity program together)
-#ifndef MG_FLOWS_NT
-#define MG_FLOWS_NT 128
-#endif
-template <class P, int NT_ = MG_FLOWS_NT>
-struct LayoutFlowsTmem {
-  static constexpr int NT = NT_;
-  static_assert(NT == 128 || NT == 256, "128 TMEM lanes, one or two column halves");
-  static constexpr size_t r128(size_t b) { return ((b + 127) / 128) * 128; }
-  static constexpr size_t bar_bytes = 128;  // TMA bar, TMEM address
-  static constexpr size_t stage_bytes = size_t(NT) * P::NPAR * 4 * sizeof(double);
-  static constexpr size_t slab_bytes = size_t(NT) * slab_slots<P, float>() * sizeof(float);
-  static constexpr size_t stage_off = bar_bytes;
-  static constexpr size_t slab_off = stage_off + r128(stage_bytes);
-  static constexpr size_t base_bytes = slab_off + r128(slab_bytes);
-  static constexpr uint32_t tmem_cols = 256 * (NT / 128);
-};
-
-template <class P>
-__global__ void __launch_bounds__(MG_FLOWS_NT)
-    flows_tmem_kernel(const double* __restrict__ mom, long long nevt, float2* __restrict__ J, long long ldj,
-                      const int* __restrict__ hels, int nhel, KParams kp, unsigned* __restrict__ status) {
-  using LY = LayoutFlowsTmem<P>;
-  constexpr int NT = LY::NT;
-  static_assert(2 * P::NCOL <= 256, "flows fit in a column half");
-  extern __shared__ __align__(128) unsigned char smem[];
-  uint64_t* tma_bar = reinterpret_cast<uint64_t*>(smem);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 16);
-  double* stage = reinterpret_cast<double*>(smem + LY::stage_off);
-  float* slab = reinterpret_cast<float*>(smem + LY::slab_off);
-  const int tid = threadIdx.x;
-  const int warp = tid >> 5;
-  const int nvalid = load_and_prepare_at<P, float, NT>(tma_bar, stage, slab, mom, nevt, kp, status);
-  if (nvalid < 0) return;
-  if (warp == 0) {
-    tc::tmem_alloc(tmem_slot, LY::tmem_cols);
-    tc::tmem_relinquish();
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
-  const FlowsTmem fl{tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(warp >> 2) * 256u};
-  const long long e = (long long)blockIdx.x * NT + tid;
-  const bool in_rows = e < ldj;  // rows are padded to 128 events, the grid to NT
-#pragma unroll 1
-  for (int ih = 0; ih < nhel; ih++) {
-    const int h = __ldg(hels + ih);
-    P::template amplitudes_store<float>(slab + tid, NT, h, kp.v, fl);
-    float2* row = J + (long long)ih * P::NCOL * ldj + e;
-#pragma unroll 1
-    for (int c = 0; c < 2 * P::NCOL; c += 16) {
-      float v[16];
-      tc::tmem_ld16(fl.taddr + (uint32_t)c, v);
-      tc::tmem_wait_ld();
-#pragma unroll
-      for (int q = 0; q < 8; q++) {
-        const int k = c / 2 + q;
-        if (k < P::NCOL && in_rows) row[(long long)k * ldj] = make_float2(v[2 * q], v[2 * q + 1]);
-      }
-    }
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) {
-    tc::fence_after_sync();
-    tc::tmem_dealloc(tmem, LY::tmem_cols);
-  }
-}
-
-// FP64 |M|^2 with the colour flows in tensor memory: 128 events per CTA,
-// four TMEM columns per flow (all 512 columns for 120 flows); shared memory
-// holds only the momenta tile and the FP64 slab, 4 warps per SM instead of 2.
-// The colour form reads the flows back from TMEM in blocks of four.
-template <class P>
-struct LayoutTmem64 {
-  static constexpr int NT = 128;
-  static constexpr size_t r128(size_t b) { return ((b + 127) / 128) * 128; }
-  static constexpr size_t bar_bytes = 128;  // TMA bar, TMEM address
-  static constexpr size_t stage_bytes = size_t(NT) * P::NPAR * 4 * sizeof(double);
-  static constexpr size_t slab_bytes = size_t(NT) * slab_slots<P, double>() * sizeof(double);
-  static constexpr size_t stage_off = bar_bytes;
-  static constexpr size_t slab_off = stage_off + r128(stage_bytes);
-  static constexpr size_t base_bytes = slab_off + r128(slab_bytes);
-  static constexpr uint32_t tmem_cols = 512;
-};
-
-// four FP64 flows (16 columns) from TMEM
-__device__ __forceinline__ void tmem_flows4(uint32_t taddr, double re[4], double im[4]) {
-  float v[16];
-  tc::tmem_ld16(taddr, v);
-  tc::tmem_wait_ld();
-#pragma unroll
-  for (int q = 0; q < 4; q++) {
-    re[q] = __hiloint2double(__float_as_int(v[4 * q + 1]), __float_as_int(v[4 * q]));
-    im[q] = __hiloint2double(__float_as_int(v[4 * q + 3]), __float_as_int(v[4 * q + 2]));
-  }
-}
-
-// sum_ij K_ij (Re J_i Re J_j + Im J_i Im J_j) from the FP64 flows in TMEM;
-// knum: K_ii on the diagonal, 2 K_ij for j > i
-template <class P>
-__device__ __forceinline__ double colour_tmem64(uint32_t taddr, const short* __restrict__ knum) {
-  static_assert(P::NCOL % 4 == 0, "blocks of four flows");
-  constexpr int NB = P::NCOL / 4;
-  double acc = 0.0;
-#pragma unroll 1
-  for (int ib = 0; ib < NB; ib++) {
-    double ri[4], ii[4], yr[4], yi[4];
-    tmem_flows4(taddr + 16u * ib, ri, ii);
-#pragma unroll
-    for (int a = 0; a < 4; a++) {
-      yr[a] = 0.0;
-      yi[a] = 0.0;
-#pragma unroll
-      for (int b = a; b < 4; b++) {
-        const double k = (double)__ldg(knum + (4 * ib + a) * P::NCOL + 4 * ib + b);
-        yr[a] = ::fma(k, ri[b], yr[a]);
-        yi[a] = ::fma(k, ii[b], yi[a]);
-      }
-    }
-#pragma unroll 1
-    for (int jb = ib + 1; jb < NB; jb++) {
-      double rj[4], ij[4];
-      tmem_flows4(taddr + 16u * jb, rj, ij);
-#pragma unroll
-      for (int a = 0; a < 4; a++)
-#pragma unroll
-        for (int b = 0; b < 4; b++) {
-          const double k = (double)__ldg(knum + (4 * ib + a) * P::NCOL + 4 * jb + b);
-          yr[a] = ::fma(k, rj[b], yr[a]);
-          yi[a] = ::fma(k, ij[b], yi[a]);
-        }
-    }
-#pragma unroll
-    for (int a = 0; a < 4; a++) acc = ::fma(ri[a], yr[a], ::fma(ii[a], yi[a], acc));
-  }
-  return acc;
-}
-
-template <class P>
-__global__ void __launch_bounds__(128, 1)
-    sigma_tmem64_kernel(const double* __restrict__ mom, long long nevt, double* __restrict__ me,
-                        const int* __restrict__ hels, int nhel, KParams kp, unsigned* __restrict__ status) {
-  using LY = LayoutTmem64<P>;
-  constexpr int NT = 128;
-  static_assert(4 * P::NCOL <= (int)LY::tmem_cols, "flows fit in the allocated columns");
-  extern __shared__ __align__(128) unsigned char smem[];
-  uint64_t* tma_bar = reinterpret_cast<uint64_t*>(smem);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 16);
-  double* stage = reinterpret_cast<double*>(smem + LY::stage_off);
-  double* slab = reinterpret_cast<double*>(smem + LY::slab_off);
-  const int tid = threadIdx.x;
-  const int warp = tid >> 5;
-  const int nvalid = load_and_prepare_at<P, double, NT>(tma_bar, stage, slab, mom, nevt, kp, status);
-  if (nvalid < 0) return;
-  if (warp == 0) {
-    tc::tmem_alloc(tmem_slot, LY::tmem_cols);
-    tc::tmem_relinquish();
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
-  const FlowsTmem64 fl{tmem + ((uint32_t)(warp * 32) << 16)};
-  const short* knum = P::knum_dev();
-  double acc = 0.0;
-#pragma unroll 1
-  for (int ih = 0; ih < nhel; ih++) {
-    const int h = __ldg(hels + ih);
-    P::template amplitudes_store<double>(slab + tid, NT, h, kp.v, fl);
-    acc += colour_tmem64<P>(fl.taddr, knum);
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) {
-    tc::fence_after_sync();
-    tc::tmem_dealloc(tmem, LY::tmem_cols);
-  }
-  if (tid < nvalid) {
-    constexpr double norm = 1.0 / (P::IDEN * P::CDEN);
-    me[(long long)blockIdx.x * NT + tid] = acc * norm;
-  }
-}
-
-template <class P>
-int launch_sigma_tmem64(const LaunchArgs& a) {
-  constexpr size_t smem = LayoutTmem64<P>::base_bytes;
-  static const cudaError_t attr = set_smem_attr(sigma_tmem64_kernel<P>, smem);
-  if (attr != cudaSuccess) return -4;
-  if (a.nevt <= 0) return 0;
-  sigma_tmem64_kernel<P><<<(unsigned)((a.nevt + 127) / 128), 128, smem, a.stream>>>(a.mom, a.nevt, a.out, a.hels,
-                                                                                     a.nhel, a.kp, a.status);
-  return cudaGetLastError() == cudaSuccess ? 0 : -4;
-}
-
-// The two phases over slices of the good helicities, every event in each
-// launch (full grids), with a stream-ordered workspace of at most
-// ROWS_WORKSPACE bytes of flows (FP32 complex [slice][NCOL][events]).
+// The stream-ordered workspace of one call: at most ROWS_WORKSPACE bytes of
+// flows (FP32 complex).
 constexpr size_t ROWS_WORKSPACE = size_t(1) << 30;
 
-// Rows per event padded to 128, and the helicities of one slice: as many as
-// fit ROWS_WORKSPACE (at least one, at most nhel).
+// Its size, in rows of one helicity over the events padded to 128: as many
+// helicities as fit ROWS_WORKSPACE (at least one, at most nhel).
 inline long long rows_ld(long long nevt) { return (nevt + 127) / 128 * 128; }
 inline long long rows_slice(int ncol, long long nevt, int nhel) {
   const size_t per_hel = (size_t)ncol * (size_t)rows_ld(nevt) * sizeof(float2);
@@ -743,61 +241,6 @@ inline long long rows_slice(int ncol, long long nevt, int nhel) {
 inline size_t rows_workspace_bytes(int ncol, long long nevt, int nhel) {
   if (nevt <= 0 || nhel <= 0) return 0;
   return (size_t)rows_slice(ncol, nevt, nhel) * (size_t)ncol * (size_t)rows_ld(nevt) * sizeof(float2);
-}
-
-template <class P, int NT>
-int launch_sigma_rows(const LaunchArgs& a) {
-  static_assert(128 % NT == 0, "flow rows are padded to 128 events");
-  constexpr bool tmem_flows = MG_FLOWS_TMEM != 0;
-  constexpr int NT1 = tmem_flows ? LayoutFlowsTmem<P>::NT : NT;
-  constexpr size_t smem1 = tmem_flows ? LayoutFlowsTmem<P>::base_bytes : Layout<P, float, NT>::base_bytes;
-  constexpr size_t smem2 = LayoutRows<P>::base_bytes;
-  static const cudaError_t attr1 = [] {
-    if constexpr (tmem_flows)
-      return set_smem_attr(flows_tmem_kernel<P>, smem1);
-    else
-      return set_smem_attr(flows_kernel<P, NT>, smem1);
-  }();
-  static const cudaError_t attr2 = set_smem_attr(colour_rows_tc_kernel<P>, smem2);
-  if (attr1 != cudaSuccess || attr2 != cudaSuccess) return -4;
-  if (a.nevt <= 0 || a.nhel <= 0) return 0;
-  const long long ldj = rows_ld(a.nevt);
-  const long long hs = rows_slice(P::NCOL, a.nevt, a.nhel);
-  float2* J = nullptr;
-  if (cudaMallocAsync(reinterpret_cast<void**>(&J), rows_workspace_bytes(P::NCOL, a.nevt, a.nhel), a.stream) !=
-      cudaSuccess)
-    return -4;
-  if (a.marks) a.marks->mark(a.stream);
-  for (int h0 = 0; h0 < a.nhel; h0 += (int)hs) {
-    const int nh = a.nhel - h0 < hs ? a.nhel - h0 : (int)hs;
-    if constexpr (tmem_flows)
-      flows_tmem_kernel<P><<<(unsigned)((a.nevt + NT1 - 1) / NT1), NT1, smem1, a.stream>>>(
-          a.mom, a.nevt, J, ldj, a.hels + h0, nh, a.kp, a.status);
-    else
-      flows_kernel<P, NT><<<(unsigned)((a.nevt + NT - 1) / NT), NT, smem1, a.stream>>>(
-          a.mom, a.nevt, J, ldj, a.hels + h0, nh, a.kp, a.status);
-    if (a.marks) a.marks->mark(a.stream);
-    colour_rows_tc_kernel<P><<<(unsigned)(ldj / 128), 128, smem2, a.stream>>>(
-        J, ldj, a.nevt, a.out, nh, h0 == 0, h0 + nh == a.nhel, static_cast<const uint4*>(a.ctile), a.status,
-        a.kp.polls);
-    if (a.marks) a.marks->mark(a.stream);
-  }
-  const cudaError_t e1 = cudaGetLastError();
-  const cudaError_t e2 = cudaFreeAsync(J, a.stream);
-  return (e1 == cudaSuccess && e2 == cudaSuccess) ? 0 : -4;
-}
-
-template <class P>
-int launch_sigma_tc(const LaunchArgs& a) {
-  constexpr int NT = 128;
-  constexpr size_t smem = LayoutTC<P, NT>::base_bytes;
-  static const cudaError_t attr = set_smem_attr(sigma_tc_kernel<P, NT>, smem);
-  if (attr != cudaSuccess) return -4;
-  if (a.nevt <= 0) return 0;
-  const long long grid = (a.nevt + NT - 1) / NT;
-  sigma_tc_kernel<P, NT><<<(unsigned)grid, NT, smem, a.stream>>>(a.mom, a.nevt, a.out, a.hels, a.nhel, a.kp,
-                                                                   static_cast<const uint4*>(a.ctile), a.status);
-  return cudaGetLastError() == cudaSuccess ? 0 : -4;
 }
 
 }  // namespace mg

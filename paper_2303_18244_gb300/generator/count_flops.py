@@ -8,6 +8,10 @@ paper_2303_18244_gb300/flops.json:
   {tag: {"amp_flops_per_hel": ..., "colour_flops_per_hel": ...,
          "colour_dense_flops_per_hel": 4 * ncol^2, "nhel": ..., "ncol": ...}}
 
+and, for the processes whose kernels run the helicity-shared recursion, the
+work of one event over all its helicities (currents, closings, colour form):
+  {"rec_flops_per_event": ..., "rec_colour_flops_per_event": ...}
+
 The counts are those of the source as generated (before any compiler
 simplification), i.e. the algorithmic work of steps A2-A5 per helicity.
 Run: python -m paper_2303_18244_gb300.generator.count_flops
@@ -68,15 +72,55 @@ int main() {
 """
 
 
-def count(tag: str) -> dict:
+# the recursion of one event with one thread, the same counting type
+PROGRAM_REC = PROGRAM[:PROGRAM.index('#include "mg_vertices.cuh"')].replace("#include <cstdio>", "#include <cstdio>\n#include <cstdlib>\n#include <vector>") + r"""
+namespace std { inline Cnt fma(Cnt a, Cnt b, Cnt c) { n_add++; n_mul++; return Cnt(a.v * b.v + c.v); } }
+#include "gen/TAG_rec.cuh"
+using namespace mg;
+using P = TAG_rec;
+using ST = rec::Store<Cnt, P::N, P::NVEC<Cnt>>;
+int main() {
+  std::vector<Cnt> mem(ST::bytes / sizeof(Cnt) + 16, Cnt(0.01));
+  const ST st(reinterpret_cast<void*>((reinterpret_cast<size_t>(mem.data()) + 15) / 16 * 16));
+  double kp[8] = {1.2, 173.0, 1.5, 0, 0, 0, 0, 0};
+  long long colour = 0;
+  CURRENTS
+  for (int hg = 0; hg < (1 << P::N); hg++)
+    for (int s = 0; s < 2; s++) {
+      static cx<Cnt> a[2][P::NCOL];
+      FLOWS
+      for (int b = 0; b < 2; b++) {
+        const long long before = n_add + n_mul;
+        volatile double v = P::colour_form<Cnt>(a[b]).v;
+        (void)v;
+        colour += n_add + n_mul - before;
+      }
+    }
+  printf("%lld %lld\n", n_add + n_mul - colour, colour);
+  return 0;
+}
+"""
+
+
+def _run(program: str) -> list[int]:
     with tempfile.TemporaryDirectory() as d:
         src = os.path.join(d, "c.cpp")
         exe = os.path.join(d, "c")
         with open(src, "w") as f:
-            f.write(PROGRAM.replace("TAG", tag))
+            f.write(program)
         subprocess.run(["g++", "-O0", "-std=c++17", f"-I{CSRC}", "-o", exe, src], check=True)
-        out = subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split()
-    amp, col, nhel, ncol = (int(x) for x in out)
+        return [int(x) for x in subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split()]
+
+
+def count_recursion(tag: str, n: int) -> dict:
+    from paper_2303_18244_gb300.generator.recursion import HOST_CURRENTS, HOST_FLOWS
+    src = PROGRAM_REC.replace("CURRENTS", HOST_CURRENTS[n > 4]).replace("FLOWS", HOST_FLOWS[n > 4])
+    amp, col = _run(src.replace("<double", "<Cnt").replace("TAG", tag))
+    return {"rec_flops_per_event": amp, "rec_colour_flops_per_event": col}
+
+
+def count(tag: str) -> dict:
+    amp, col, nhel, ncol = _run(PROGRAM.replace("TAG", tag))
     return {"amp_flops_per_hel": amp, "colour_flops_per_hel": col,
             "colour_dense_flops_per_hel": 4 * ncol * ncol, "nhel": nhel, "ncol": ncol}
 
@@ -85,7 +129,7 @@ def main(tags=None):
     sys.path.insert(0, os.path.dirname(PKG))
     from paper_2303_18244_gb300 import build as B
     B.generate()
-    from paper_2303_18244_gb300.generator.emit import PROCESSES
+    from paper_2303_18244_gb300.generator.emit import PROCESSES, RECURSION
     tags = tags or [t for t, _ in PROCESSES.values()]
     res = {}
     if os.path.exists(OUT):
@@ -93,6 +137,8 @@ def main(tags=None):
             res = json.load(f)
     for t in tags:
         res[t] = count(t)
+        if t in RECURSION["f64"]:
+            res[t].update(count_recursion(t, next(n for q, n in PROCESSES.values() if q == t)))
         print(t, res[t])
     with open(OUT, "w") as f:
         json.dump(res, f, indent=1, sort_keys=True)

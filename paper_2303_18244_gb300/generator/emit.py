@@ -309,13 +309,6 @@ def emit_gg(n: int, tag: str, mode: str = "straight", chunk_order: str = "patter
     # product V.J (gg -> t t~ g g: 74 pairs for 114 amplitudes, measured 6 %
     # faster in FP32, 11 % in FP64; MG_PAIR_V=0 turns it off)
     pair_v = os.environ.get("MG_PAIR_V", "1") == "1"
-    # chunked mode, MG_FLUSH_CALL=1: a colour pattern's flows are updated by one
-    # non-inlined call over its entry in a device table of (flow << 1 | minus)
-    # instead of inline code per pattern (gg -> t t~ g g g: measured 2.5x
-    # slower in FP32, 15 % in FP64)
-    flush_calls = os.environ.get("MG_FLUSH_CALL", "0") == "1"
-    flow_list: list = []
-    flow_list_off: dict = {}
     pair_uses: dict = {}
     for ai in amp_order:
         op = plan.amps[ai][0]
@@ -351,14 +344,7 @@ def emit_gg(n: int, tag: str, mode: str = "straight", chunk_order: str = "patter
             L.append(f"    pacc = pacc {'+' if psign[ai] > 0 else '-'} a;")
             if last_of[pid[ai]] == ai:
                 pat = pats[pid[ai]]
-                if mode == "chunked" and flush_calls:
-                    # the pattern's flow list in the device table; one call
-                    off = flow_list_off.setdefault(pid[ai], len(flow_list))
-                    if off == len(flow_list):
-                        flow_list.extend((k << 1) | (1 if c < 0 else 0) for k, c in pat)
-                    L.append(f"    jamp.flush({tag}_FLOWLIST + {off}, {len(pat)}, pacc);")
-                    L.append("    pacc = cx<R>{R(0), R(0)};")
-                elif mode == "chunked":
+                if mode == "chunked":
                     kk = ", ".join(str(k) for k, _ in pat)
                     sg = ", ".join("1" if c > 0 else "-1" for _, c in pat)
                     L.append(f"    {{ constexpr int kk[{len(pat)}] = {{{kk}}}; constexpr int sg[{len(pat)}] = {{{sg}}};")
@@ -477,7 +463,6 @@ def emit_gg(n: int, tag: str, mode: str = "straight", chunk_order: str = "patter
         L.append(f"static constexpr int NCHUNK = {len(chunks)};")
         L.append(f"static constexpr int NSTORE = {nstore};")
         L.append("// one helicity: the chunks in order, the colour flows in the store J")
-        L.append("// (FlowsSmem: shared memory; FlowsTmem: tensor memory)")
         L.append("template <typename R, typename J>")
         L.append("__device__ static __forceinline__ void amplitudes_store(const R* __restrict__ ev, const int es, "
                  "const int hel, const double* __restrict__ kp, const J jamp) {")
@@ -485,8 +470,6 @@ def emit_gg(n: int, tag: str, mode: str = "straight", chunk_order: str = "patter
         L.append("  jamp.zero(NCOL);")
         for j in range(len(chunks)):
             L.append(f"  chunk{j}<R, J>(ev, es, hel, kp, W, jamp);")
-            if j + 1 < len(chunks):
-                L.append("  jamp.chunk_done();")
         L.append("}")
         L.append("template <typename R>")
         L.append("__device__ static __forceinline__ void amplitudes(const R* __restrict__ ev, const int es, const int hel,")
@@ -501,9 +484,6 @@ def emit_gg(n: int, tag: str, mode: str = "straight", chunk_order: str = "patter
         src = "\n".join(L) + "\n"
         src = src.replace('#include "mg_vertices.cuh"', '#include "mg_vertices.cuh"\n#include "mg_flowstore.cuh"', 1)
         tables = _knum_table(tag, K)
-        if flush_calls:
-            tables += (f"\nstatic __device__ const short {tag}_FLOWLIST[{max(1, len(flow_list))}] = {{"
-                       + ", ".join(str(v) for v in flow_list) + "};")
         return src.replace(f"struct {tag} {{", tables + f"\nstruct {tag} {{", 1)
 
     if group:
@@ -1196,21 +1176,6 @@ THREADS = {
 }
 
 
-# processes whose mixed path contracts colour on the tensor cores (the FP16
-# operand tiles of 128 events plus FP32 colour-flow accumulators must fit in
-# shared memory next to the per-event slab)
-TENSOR_CORE_COLOUR = {"ggttg", "ggttgg"}
-# tensor-core processes whose colour flows share the operand tiles' space
-TC_ALIAS = {"ggttgg"}
-# processes whose FP64 |M|^2 keeps the colour flows in tensor memory (120
-# complex FP64 flows per event do not fit in shared memory beside the slab)
-TMEM_FP64 = set(filter(None, os.environ.get("MG_TMEM_FP64", "ggttggg").split(",")))
-# processes whose mixed path writes the colour flows of every (helicity, event)
-# row to HBM and contracts them on the tensor cores in a second kernel
-# (120 flows: the operand tiles do not fit beside the per-event state)
-TENSOR_CORE_ROWS = set(filter(None, os.environ.get("MG_TC_ROWS", "ggttggg").split(",")))
-
-
 # processes whose vertex routines are called rather than inlined, per
 # precision: the straight-line helicity program then shrinks to a sequence of
 # calls to a few small routines that stay in the instruction cache.  Measured:
@@ -1219,6 +1184,19 @@ TENSOR_CORE_ROWS = set(filter(None, os.environ.get("MG_TC_ROWS", "ggttggg").spli
 # gg -> t t~ g g g 1.05e4 inlined against 8.4e3 called) and the smaller
 # processes keep the inlined code
 VERTEX_CALLS = {"f32": {"ggttgg", "ggttggg"}, "f64": set()}
+
+
+# processes whose kernels run the helicity-shared recursion (recursion.py), by
+# the arithmetic of the amplitudes.  FP32 covers MG_MIXED and MG_FLOAT, FP64
+# every other mode; the helicity and colour choice of the FP32 modes keeps the
+# per-helicity program, whose choices must not move with the rounding of the
+# flows.  gg -> t t~ in FP32 keeps it too: sixteen short helicities of one
+# thread per event beat the recursion's small stages (524288 events 0.20
+# against 0.58 ms; FP64, bound by the FP64 pipe, 1.17 against 0.69 ms per 65536).
+RECURSION = {"f32": {"ggttg", "ggttgg", "ggttggg"}, "f64": {"ggtt", "ggttg", "ggttgg", "ggttggg"}}
+# of these, the mixed mode writes the flows to a workspace and contracts colour
+# on the tensor cores in a second kernel (120 flows)
+RECURSION_ROWS = {"ggttggg"}
 
 
 # colour-flow counts of the processes written by hand (gg processes: n!)
@@ -1233,53 +1211,53 @@ def emit_tu(proc: str, prec: str) -> tuple[str, str]:
     tag, n = PROCESSES[proc]
     nt64, nt32 = THREADS[tag]
     calls = "#define MG_VERTEX __noinline__\n" if tag in VERTEX_CALLS[prec] else ""
-    if prec == "f32" and tag in TC_ALIAS:
-        calls += "#define MG_TC_ALIAS 1\n"
     head = f"// generated by paper_2303_18244_gb300.generator: {prec} kernels of '{proc}'\n{calls}"
-    tc = tag in TENSOR_CORE_COLOUR or tag in TENSOR_CORE_ROWS
+    rec = tag in RECURSION[prec]
+    rows = tag in RECURSION_ROWS
+    inc = f'#include "../mg_recursion_kernels.cuh"\n#include "{tag}_rec.cuh"\n' if rec else ""
+    # the per-helicity program (nothing of the recursion's FP64 unit runs it)
+    prog = "" if prec == "f64" and rec else f'#include "{header_name(proc, prec)}"\n'
     if prec == "f32":
-        if tag in TENSOR_CORE_ROWS:
-            mixed = f"launch_sigma_rows<{tag}, {nt32}>(a)"
-        elif tc:
-            mixed = f"launch_sigma_tc<{tag}>(a)"
+        if rec:
+            mixed = f"launch_rec_rows<{tag}_rec>(a)" if rows else f"launch_rec<{tag}_rec, float, double, double>(a)"
+            flt = f"launch_rec<{tag}_rec, float, float, float>(a)"
         else:
             mixed = f"launch_sigma<{tag}, float, {nt32}>(a)"
-        inc = '#include "../mg_colour_tc.cuh"\n' if tc else ""
+            flt = f"launch_sigma<{tag}, float, {nt32}, float, float>(a)"
         src = f"""{head}#include "../mg_kernels.cuh"
-{inc}#include "{header_name(proc, "f32")}"
-
+{inc}{prog}
 namespace mg {{
 int sigma_{tag}_mixed(const LaunchArgs& a) {{ return {mixed}; }}
 int select_{tag}_mixed(const LaunchArgs& a) {{ return launch_select<{tag}, float, {nt32}>(a); }}
-int sigma_{tag}_float(const LaunchArgs& a) {{ return launch_sigma<{tag}, float, {nt32}, float, float>(a); }}
+int sigma_{tag}_float(const LaunchArgs& a) {{ return {flt}; }}
 }}  // namespace mg
 """
         return tag, src
-    ncol = FIXED_NCOL.get(tag) or math.factorial(n)
-    tck = ((ncol + 15) // 16) * 16 if tc else 0
-    if tag in TMEM_FP64:
-        inc64 = '#include "../mg_colour_tc.cuh"\n'
-        fp64 = f"launch_sigma_tmem64<{tag}>(a)"
+    if rec:
+        fp64, hel, sel, paper = (f"launch_rec<{tag}_rec, double, double, double, {m}>(a)"
+                                 for m in ("REC_SIGMA", "REC_HELICITIES", "REC_SELECT", "REC_PAPER"))
     else:
-        inc64 = ""
-        fp64 = f"launch_sigma<{tag}, double, {nt64}>(a)"
+        fp64, hel, sel, paper = (f"launch_sigma<{tag}, double, {nt64}>(a)", f"launch_helicities<{tag}, {nt64}>(a)",
+                                 f"launch_select<{tag}, double, {nt64}>(a)", f"launch_sigma_paper<{tag}, {nt64}>(a)")
+    ncol = FIXED_NCOL.get(tag) or math.factorial(n)
+    tck = ((ncol + 15) // 16) * 16 if rows else 0
+    c = f"{tag}_rec" if rec else tag
     src = f"""{head}#include "../mg_kernels.cuh"
-{inc64}#include "{header_name(proc, "f64")}"
-
+{inc}{prog}
 namespace mg {{
 static int sigma_fp64(const LaunchArgs& a) {{ return {fp64}; }}
-static int helicities(const LaunchArgs& a) {{ return launch_helicities<{tag}, {nt64}>(a); }}
-static int select_fp64(const LaunchArgs& a) {{ return launch_select<{tag}, double, {nt64}>(a); }}
-static int paper(const LaunchArgs& a) {{ return launch_sigma_paper<{tag}, {nt64}>(a); }}
+static int helicities(const LaunchArgs& a) {{ return {hel}; }}
+static int select_fp64(const LaunchArgs& a) {{ return {sel}; }}
+static int paper(const LaunchArgs& a) {{ return {paper}; }}
 int sigma_{tag}_mixed(const LaunchArgs& a);
 int select_{tag}_mixed(const LaunchArgs& a);
 int sigma_{tag}_float(const LaunchArgs& a);
-static_assert({tag}::NCOL == {ncol}, "colour-flow count");
-static const ProcDesc desc = {{"{proc}", "{tag}", {tag}::NPAR, {tag}::NHEL, {tag}::NCOL, {tag}::NDIAG,
-                              {tag}::NAMP, {tag}::IDEN, {tag}::CDEN, {tag}::KNUM,
+static_assert({c}::NCOL == {ncol}, "colour-flow count");
+static const ProcDesc desc = {{"{proc}", "{tag}", {c}::NPAR, {c}::NHEL, {c}::NCOL, {c}::NDIAG,
+                              {c}::NAMP, {c}::IDEN, {c}::CDEN, {c}::KNUM,
                               sigma_fp64, sigma_{tag}_mixed, helicities, {tck},
                               select_fp64, select_{tag}_mixed, paper, sigma_{tag}_float,
-                              {1 if tag in TENSOR_CORE_ROWS else 0}}};
+                              {f"{tag}_rec::KNUM_ORDERED" if rows else "nullptr"}, {1 if rows else 0}}};
 const ProcDesc* proc_{tag}() {{ return &desc; }}
 }}  // namespace mg
 """
