@@ -20,8 +20,6 @@
 
 namespace {
 
-constexpr int MAX_FINAL = 5;
-
 __device__ __forceinline__ void philox4x64_10(uint64_t c[4], uint64_t k0, uint64_t k1) {
   const uint64_t M0 = 0xD2E7470EE14C6C93ull, M1 = 0xCA5A826395121157ull;
   const uint64_t W0 = 0x9E3779B97F4A7C15ull, W1 = 0xBB67AE8584CAA73Bull;
@@ -39,86 +37,156 @@ __device__ __forceinline__ void philox4x64_10(uint64_t c[4], uint64_t k0, uint64
   }
 }
 
-__device__ __forceinline__ double to_unit(uint64_t w) {
-  return ((double)(w >> 11) + 0.5) * 0x1.0p-53;
-}
-
 struct PSArgs {
   double sqrt_s;
   uint64_t seed;
   long long first_event, nevt;
-  int nf;
-  double mass[MAX_FINAL];
+  double mass;  // of the first two final states
+  double mu2;   // (mass / sqrt_s)^2
+  double xi0;   // sqrt(1 - (sum of the masses / sqrt_s)^2): start of the scale
 };
 
+// One event per thread, everything in registers (NF final states, a template
+// parameter).  The FP64 pipe bounds it (16 cycles per warp instruction and
+// SM): about 530 FP64 instructions per event for NF = 4.  The map works on
+// momenta in units of the generated mass M and solves for X = (scale) /
+// sqrt_s in f(X) = sum_j sqrt(mu_j^2 + X^2 |p_j|^2) - 1 = 0:
+//   - Newton in FP32 first, which leaves about 1e-7;
+//   - then FP64 steps with the FP32 derivative, each of which gains those
+//     seven digits again; a step below 1e-9 of X leaves less than the rounding
+//     of f, so two steps are usual (at most 60).
+// Newton in FP64 alone, until a step fell below 1e-16 of X, took as many
+// iterations as the slowest lane of the warp needed to meet a bound below the
+// rounding of f (up to all 60): 524288 events of NF = 4 5.66 ms.
+template <int NF, bool ALIGNED>
 __global__ void __launch_bounds__(128) rambo_kernel(PSArgs a, double* __restrict__ out) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= a.nevt) return;
   const long long ev = a.first_event + i;
-  const int nf = a.nf;
-  double q[MAX_FINAL][4];
-  for (int j = 0; j < nf; j++) {
+  double q[NF][4];
+#pragma unroll
+  for (int j = 0; j < NF; j++) {
     uint64_t c[4] = {(uint64_t)ev, (uint64_t)j, 0ull, 0ull};
     philox4x64_10(c, a.seed, 0ull);
-    const double u0 = to_unit(c[0]), u1 = to_unit(c[1]), u2 = to_unit(c[2]), u3 = to_unit(c[3]);
-    const double ct = 2.0 * u0 - 1.0;
-    const double st = sqrt(fmax(0.0, 1.0 - ct * ct));
-    const double phi = 2.0 * 3.14159265358979323846 * u1;
-    const double q0 = -log(u2 * u3);
+    // u = v 2^-53 with v = (w >> 11) + 0.5; scaling by powers of two is exact
+    const double v0 = (double)(c[0] >> 11) + 0.5, v1 = (double)(c[1] >> 11) + 0.5;
+    const double v2 = (double)(c[2] >> 11) + 0.5, v3 = (double)(c[3] >> 11) + 0.5;
+    const double ct = ::fma(v0, 0x1.0p-52, -1.0);  // 2 u0 - 1
+    const double st = sqrt(fmax(0.0, ::fma(-ct, ct, 1.0)));
+    double sn, cs;
+    sincospi(v1 * 0x1.0p-52, &sn, &cs);  // azimuth 2 pi u1
+    const double q0 = -log(v2 * v3 * 0x1.0p-106);
+    const double qt = q0 * st;
     q[j][0] = q0;
-    q[j][1] = q0 * st * cos(phi);
-    q[j][2] = q0 * st * sin(phi);
+    q[j][1] = qt * cs;
+    q[j][2] = qt * sn;
     q[j][3] = q0 * ct;
   }
   double Q[4] = {0, 0, 0, 0};
-  for (int j = 0; j < nf; j++)
+#pragma unroll
+  for (int j = 0; j < NF; j++)
+#pragma unroll
     for (int mu = 0; mu < 4; mu++) Q[mu] += q[j][mu];
   const double M = sqrt(Q[0] * Q[0] - (Q[1] * Q[1] + Q[2] * Q[2] + Q[3] * Q[3]));
-  const double b[3] = {-Q[1] / M, -Q[2] / M, -Q[3] / M};
-  const double gam = Q[0] / M;
-  const double aa = 1.0 / (1.0 + gam);
-  const double x = a.sqrt_s / M;
-  double p[MAX_FINAL][4];
-  for (int j = 0; j < nf; j++) {
-    const double bq = b[0] * q[j][1] + b[1] * q[j][2] + b[2] * q[j][3];
-    p[j][0] = x * (gam * q[j][0] + bq);
-    for (int k = 0; k < 3; k++) p[j][k + 1] = x * (q[j][k + 1] + b[k] * q[j][0] + aa * bq * b[k]);
-  }
-  // residual 3-momentum of the map removed evenly
+  const double im = 1.0 / M;
+  const double b[3] = {-Q[1] * im, -Q[2] * im, -Q[3] * im};
+  const double aa = 1.0 / ::fma(Q[0], im, 1.0);
+  // 3-momenta in the centre-of-mass frame, in units of M / sqrt_s
   double R3[3] = {0, 0, 0};
-  for (int j = 0; j < nf; j++)
-    for (int k = 0; k < 3; k++) R3[k] += p[j][k + 1];
-  for (int j = 0; j < nf; j++)
-    for (int k = 0; k < 3; k++) p[j][k + 1] -= R3[k] / nf;
-  // common 3-momentum scale xi onto the mass shells (Newton)
-  double p3sq[MAX_FINAL], msum = 0.0;
-  for (int j = 0; j < nf; j++) {
-    p3sq[j] = p[j][1] * p[j][1] + p[j][2] * p[j][2] + p[j][3] * p[j][3];
-    msum += a.mass[j];
-  }
-  double xi = sqrt(1.0 - (msum / a.sqrt_s) * (msum / a.sqrt_s));
-  for (int it = 0; it < 60; it++) {
-    double f = -a.sqrt_s, df = 0.0;
-    for (int j = 0; j < nf; j++) {
-      const double e = sqrt(a.mass[j] * a.mass[j] + xi * xi * p3sq[j]);
-      f += e;
-      df += xi * p3sq[j] / e;
+#pragma unroll
+  for (int j = 0; j < NF; j++) {
+    const double bq = b[0] * q[j][1] + b[1] * q[j][2] + b[2] * q[j][3];
+    const double w = ::fma(aa, bq, q[j][0]);
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      q[j][k + 1] = ::fma(b[k], w, q[j][k + 1]);
+      R3[k] += q[j][k + 1];
     }
-    const double step = f / df;
-    xi -= step;
-    if (fabs(step) <= 1e-16 * fabs(xi)) break;
   }
-  double* o = out + i * (long long)(nf + 2) * 4;
-  const double E = 0.5 * a.sqrt_s;
-  o[0] = E; o[1] = 0.0; o[2] = 0.0; o[3] = E;
-  o[4] = E; o[5] = 0.0; o[6] = 0.0; o[7] = -E;
-  for (int j = 0; j < nf; j++) {
-    double* t = o + 8 + 4 * j;
-    t[1] = p[j][1] * xi;
-    t[2] = p[j][2] * xi;
-    t[3] = p[j][3] * xi;
-    t[0] = sqrt(a.mass[j] * a.mass[j] + xi * xi * p3sq[j]);
+  // the map's residual 3-momentum removed evenly
+  double p2[NF], root[NF];
+  float p2f[NF];
+  double S = 0.0;  // sum of the massless |p|
+#pragma unroll
+  for (int j = 0; j < NF; j++) {
+#pragma unroll
+    for (int k = 0; k < 3; k++) q[j][k + 1] = ::fma(R3[k], -1.0 / NF, q[j][k + 1]);
+    p2[j] = q[j][1] * q[j][1] + q[j][2] * q[j][2] + q[j][3] * q[j][3];
+    p2f[j] = (float)p2[j];
+    if (j >= 2) {
+      root[j] = sqrt(p2[j]);
+      S += root[j];
+    }
   }
+  // common scale onto the mass shells
+  const double x0 = a.xi0 * im;
+  const float mu2f = (float)a.mu2, Sf = (float)S;
+  float xf = (float)x0, dinv = 0.f;
+#pragma unroll 1
+  for (int it = 0; it < 6; it++) {
+    float f = fmaf(xf, Sf, -1.f), df = Sf;
+#pragma unroll
+    for (int j = 0; j < 2; j++) {
+      const float r = rsqrtf(fmaf(xf * xf, p2f[j], mu2f));
+      f = fmaf(fmaf(xf * xf, p2f[j], mu2f), r, f);
+      df = fmaf(xf * p2f[j], r, df);
+    }
+    dinv = 1.f / df;
+    xf = fmaf(-f, dinv, xf);
+  }
+  double X = (double)xf;
+  if (!(xf > 0.f) || !(xf < 1e30f) || !(dinv > 0.f) || !(dinv < 1e30f)) X = x0;  // FP32 did not converge
+#pragma unroll 1
+  for (int it = 0; it < 60; it++) {
+    double f = ::fma(X, S, -1.0), df = S;
+    const double X2 = X * X;
+    const float Xf = (float)X;
+    float dm = Sf;
+#pragma unroll
+    for (int j = 0; j < 2; j++) {
+      const double e = sqrt(::fma(X2, p2[j], a.mu2));
+      f += e;
+      dm = fmaf(Xf * p2f[j], 1.f / (float)e, dm);
+    }
+    df = (double)(1.f / dm);
+    if (!(dm > 1e-30f) || !(dm < 1e30f)) {  // outside the FP32 range: the derivative in FP64
+      df = S;
+      for (int j = 0; j < 2; j++) df += X * p2[j] / sqrt(::fma(X2, p2[j], a.mu2));
+      df = 1.0 / df;
+    }
+    const double step = f * df;
+    X -= step;
+    if (fabs(step) <= 1e-9 * fabs(X)) break;
+  }
+  double* o = out + i * (long long)(NF + 2) * 4;
+  auto put = [&](int slot, double e, double x, double y, double z) {
+    double* t = o + 4 * slot;
+    if constexpr (ALIGNED) {
+      reinterpret_cast<double2*>(t)[0] = make_double2(e, x);
+      reinterpret_cast<double2*>(t)[1] = make_double2(y, z);
+    } else {
+      t[0] = e;
+      t[1] = x;
+      t[2] = y;
+      t[3] = z;
+    }
+  };
+  const double E = 0.5 * a.sqrt_s, scale = X * a.sqrt_s, m2 = a.mass * a.mass;
+  put(0, E, 0.0, 0.0, E);
+  put(1, E, 0.0, 0.0, -E);
+#pragma unroll
+  for (int j = 0; j < NF; j++)
+    put(2 + j, j < 2 ? sqrt(::fma(scale * scale, p2[j], m2)) : scale * root[j], scale * q[j][1], scale * q[j][2],
+        scale * q[j][3]);
+}
+
+template <int NF>
+void launch_rambo(const PSArgs& a, double* out, cudaStream_t s) {
+  const unsigned grid = (unsigned)((a.nevt + 127) / 128);
+  if ((reinterpret_cast<uintptr_t>(out) & 15u) == 0)
+    rambo_kernel<NF, true><<<grid, 128, 0, s>>>(a, out);
+  else
+    rambo_kernel<NF, false><<<grid, 128, 0, s>>>(a, out);
 }
 
 }  // namespace
@@ -133,19 +201,26 @@ extern "C" int mg_rambo(const mg_process* h, double sqrt_s, uint64_t seed, int64
   a.seed = seed;
   a.first_event = first_event;
   a.nevt = nevt;
-  a.nf = h->d->npar - 2;
-  if (a.nf < 2 || a.nf > MAX_FINAL) return MG_ERR_ARG;
+  const int nf = h->d->npar - 2;
+  if (nf < 2 || nf > 5) return MG_ERR_ARG;
   // final-state masses: the top pair of g g -> t t~ (+ gluons); massless leptons
   const bool tops = std::strcmp(h->d->tag, "eemumu") != 0;
-  for (int j = 0; j < a.nf; j++) a.mass[j] = (tops && j < 2) ? h->par.mt : 0.0;
-  double msum = 0.0;
-  for (int j = 0; j < a.nf; j++) msum += a.mass[j];
-  if (msum >= sqrt_s) return MG_ERR_ARG;
+  a.mass = tops ? h->par.mt : 0.0;
+  if (2.0 * a.mass >= sqrt_s) return MG_ERR_ARG;
+  a.mu2 = (a.mass / sqrt_s) * (a.mass / sqrt_s);
+  a.xi0 = std::sqrt(1.0 - (2.0 * a.mass / sqrt_s) * (2.0 * a.mass / sqrt_s));
   int prev = -1, dev = h->device;
   cudaGetDevice(&prev);
   if (prev != dev) cudaSetDevice(dev);
-  const long long grid = (nevt + 127) / 128;
-  rambo_kernel<<<(unsigned)grid, 128, 0, static_cast<cudaStream_t>(stream)>>>(a, momenta_dev);
+  const cudaStream_t cs = static_cast<cudaStream_t>(stream);
+  if (nf == 2)
+    launch_rambo<2>(a, momenta_dev, cs);
+  else if (nf == 3)
+    launch_rambo<3>(a, momenta_dev, cs);
+  else if (nf == 4)
+    launch_rambo<4>(a, momenta_dev, cs);
+  else
+    launch_rambo<5>(a, momenta_dev, cs);
   const cudaError_t e = cudaGetLastError();
   if (prev >= 0 && prev != dev) cudaSetDevice(prev);
   return e == cudaSuccess ? MG_OK : MG_ERR_CUDA;
