@@ -5,16 +5,16 @@
 // that follow the matrix element in the event generator, and names it as a
 // candidate to offload to the GPU.  Event i is kept when r_i * w_max < w_i
 // (r_i uniform in [0, 1)); the kept indices are written in increasing order,
-// so the result does not depend on the launch configuration.  Three launches:
+// so the result does not depend on the launch configuration.  Two launches:
 // per tile of 4096 events, the accept bits (one warp ballot per 32 events,
-// n/8 bytes in all) and their count; one scan of the tile counts; then each
-// tile ranks its kept events from its bits alone and writes their indices at
-// its tile's offset.  w and r are read once: 16 bytes per event, plus 8 per
-// kept index.
+// n/8 bytes in all) and their count; then a warp per tile ranks its kept events
+// from its bits alone and writes their indices behind the kept events of the
+// tiles before it, whose counts its block adds up for itself (past 16384 tiles
+// a scan of the counts in between).  w and r are read once: 16 bytes per event,
+// plus 8 per kept index; bound by HBM.
 #include <cuda_runtime.h>
 
 #include "mg.h"
-#include "mg_kernels.cuh"  // mbarrier and bulk-copy primitives
 
 // MG_UW_FP32_FIRST (default 1): the decision r_i * w_max < w_i is taken in
 // FP32 where the FP32 values are far enough apart to make it certain, in FP64
@@ -23,12 +23,6 @@
 // FP32); the kept set is the same bit for bit.
 #ifndef MG_UW_FP32_FIRST
 #define MG_UW_FP32_FIRST 1
-#endif
-// MG_UW_TMA: the count pass takes each full tile of 16-byte aligned w and r
-// into shared memory with two bulk copies (TMA engine) instead of per-thread
-// loads.
-#ifndef MG_UW_TMA
-#define MG_UW_TMA 0
 #endif
 
 namespace {
@@ -75,7 +69,7 @@ __device__ __forceinline__ bool kept_exact(double r, double w, double w_max, flo
   return r * w_max < w;
 }
 
-// Pass 1.  Thread t of tile b takes events b*TILE + j*THREADS + t, j < PER_THREAD
+// First pass.  Thread t of tile b takes events b*TILE + j*THREADS + t, j < PER_THREAD
 // (coalesced); word j*WARPS + warp of the tile's bits holds the ballot of
 // events b*TILE + j*THREADS + warp*32 + lane, so the words in order cover the
 // tile in increasing index order.
@@ -113,74 +107,7 @@ __global__ void __launch_bounds__(UW_THREADS)
   }
 }
 
-// Pass 1 with the tile staged by the TMA engine: one thread issues two bulk
-// copies (w and r of the tile, 2 x 8 * TILE bytes) that complete on one
-// mbarrier, then every thread reads its events from shared memory; events,
-// bit words and counts as in tile_count_kernel.  Full tiles only, with w and
-// r 16-byte aligned (checked on the host); the partial last tile takes
-// per-thread loads.  A copy that does not complete within the bounded wait
-// is waited for once more (bounded), so that none is left in flight, and the
-// tile is then read from global memory.
-constexpr size_t UW_TMA_SMEM = 128 + 2 * sizeof(double) * UW_TILE;
-
-__global__ void __launch_bounds__(UW_THREADS)
-    tile_count_tma_kernel(const double* __restrict__ w, const double* __restrict__ r, long long n, double w_max,
-                          long long* __restrict__ counts, unsigned* __restrict__ bits) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ int warp_sum[UW_WARPS];
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
-  double* sw = reinterpret_cast<double*>(smem + 128);
-  double* sr = sw + UW_TILE;
-  const long long base = (long long)blockIdx.x * UW_TILE;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned* tb = bits + (long long)blockIdx.x * UW_WORDS;
-  float wmf = 0.f;
-  const bool wm_ok = f32_trunc(w_max, wmf);
-  bool staged = false;
-  if (base + UW_TILE <= n) {  // uniform across the CTA
-    if (threadIdx.x == 0) {
-      mg::mbar_init(bar, 1);
-      mg::fence_mbar_init();
-      mg::fence_proxy_async_smem();
-      mg::mbar_arrive_expect_tx(bar, (uint32_t)(2 * sizeof(double) * UW_TILE));
-      mg::bulk_g2s(sw, w + base, (uint32_t)(sizeof(double) * UW_TILE), bar);
-      mg::bulk_g2s(sr, r + base, (uint32_t)(sizeof(double) * UW_TILE), bar);
-    }
-    __syncthreads();
-    staged = __syncthreads_and(mg::mbar_wait_bounded(bar, 0, mg::WAIT_POLLS) ? 1 : 0) != 0;
-    if (!staged) mg::mbar_wait_bounded(bar, 0, mg::WAIT_POLLS);
-  }
-  double wv[UW_PER_THREAD], rv[UW_PER_THREAD];
-#pragma unroll
-  for (int j = 0; j < UW_PER_THREAD; j++) {
-    const int k = j * UW_THREADS + threadIdx.x;
-    const long long i = base + k;
-    if (staged) {
-      wv[j] = sw[k];
-      rv[j] = sr[k];
-    } else {
-      wv[j] = i < n ? __ldcs(w + i) : 0.0;
-      rv[j] = i < n ? __ldcs(r + i) : 1.0;
-    }
-  }
-  int c = 0;
-#pragma unroll
-  for (int j = 0; j < UW_PER_THREAD; j++) {
-    const long long i = base + j * UW_THREADS + threadIdx.x;
-    const unsigned m = __ballot_sync(0xffffffffu, i < n && kept_exact(rv[j], wv[j], w_max, wmf, wm_ok));
-    if (lane == 0) tb[j * UW_WARPS + warp] = m;
-    c += __popc(m);
-  }
-  if (lane == 0) warp_sum[warp] = c;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    long long t = 0;
-    for (int k = 0; k < UW_WARPS; k++) t += warp_sum[k];
-    counts[blockIdx.x] = t;
-  }
-}
-
-// Pass 2: exclusive scan of the tile counts in place, by one block, in
+// Many tiles: exclusive scan of the tile counts in place, by one block, in
 // passes of SCAN_T * SCAN_V tiles: thread t of warp w holds the tiles
 // base + j*SCAN_T + t (j < SCAN_V; coalesced loads and stores), so the
 // (j, w, lane) order is the index order.  Warp scans of each j, one scan of
@@ -238,48 +165,102 @@ __global__ void __launch_bounds__(SCAN_T) tile_scan_kernel(long long* __restrict
   if (t == 0) *n_acc = carry;
 }
 
-// Pass 3: from the tile's bits only, each kept event's rank in the tile (the
-// counts of the words before its word, then the bits below its lane) and its
-// index at the tile's offset.  A tile without kept events (its offset equal
-// to the next tile's, or to the total for the last tile) returns at once.
+// Last pass: a warp per tile, WRITE_TILES tiles per block.  The kept events
+// before the block's first tile: SCANNED, from the scan; otherwise the block
+// adds up the counts of all earlier tiles (ntiles^2 / 4 bytes of L2 reads over
+// all blocks, 67 MB at SUM_TILES tiles, about what the scan of one block and
+// its launch cost there).  33.6 M events, 2.7 % kept: count 78 + scan 8 + a
+// block per tile 22 us before; count 78 + write 9 us now, 111.8 -> 92.4 us a
+// call; 8 / 16 / 32 tiles per block 91.9 / 92.4 / 93.2 us; without the early
+// launch 96.4 us.
+// Lane l takes words l*WPL .. of the tile, consecutive events; a tile with few
+// kept events writes them lane by lane, a fuller one word by word (coalesced).
+constexpr int WRITE_TILES = 16;
+constexpr long long SUM_TILES = 16384;
+
+template <bool SCANNED>
 __global__ void __launch_bounds__(UW_THREADS)
-    tile_write_kernel(const unsigned* __restrict__ bits, const long long* __restrict__ offsets,
-                      const long long* __restrict__ n_acc, long long* __restrict__ idx_out) {
-  constexpr int WPL = UW_WORDS / 32;  // words per lane in the word scan
-  static_assert(UW_WORDS % 32 == 0, "whole warps of words");
-  __shared__ int word_excl[UW_WORDS];
-  const long long base = (long long)blockIdx.x * UW_TILE;
+    tile_write_kernel(const unsigned* __restrict__ bits, const long long* __restrict__ counts, long long ntiles,
+                      long long* __restrict__ n_acc, long long* __restrict__ idx_out) {
+  constexpr int WPL = UW_WORDS / 32;               // words per lane
+  constexpr int PER_WARP = WRITE_TILES / UW_WARPS;  // tiles per warp
+  static_assert(UW_WORDS % 32 == 0 && WRITE_TILES <= 32, "whole warps of words, at most one tile count per lane");
+  __shared__ long long part[UW_WARPS], first[WRITE_TILES];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned* tb = bits + (long long)blockIdx.x * UW_WORDS;
-  const long long off = offsets[blockIdx.x];
-  const long long next = blockIdx.x + 1 < gridDim.x ? offsets[blockIdx.x + 1] : *n_acc;
-  if (next == off) return;  // the same for every thread of the tile
-  if (warp == 0) {
-    // words q*32 + lane in index order: a warp scan per block of 32 words,
-    // carried over the blocks
-    int cnt[WPL];
+  const long long t0 = (long long)blockIdx.x * WRITE_TILES;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // launched while the pass before it drains
+  unsigned m[PER_WARP][WPL];
 #pragma unroll
-    for (int q = 0; q < WPL; q++) cnt[q] = __popc(tb[q * 32 + lane]);
-    int carry = 0;
+  for (int k = 0; k < PER_WARP; k++) {
+    const long long t = t0 + warp * PER_WARP + k;
 #pragma unroll
-    for (int q = 0; q < WPL; q++) {
-      int sc = cnt[q];
+    for (int q = 0; q < WPL; q++) m[k][q] = t < ntiles ? bits[t * UW_WORDS + lane * WPL + q] : 0u;
+  }
+  if constexpr (SCANNED) {
+    if (threadIdx.x < WRITE_TILES) first[threadIdx.x] = t0 + threadIdx.x < ntiles ? counts[t0 + threadIdx.x] : 0;
+    __syncthreads();
+  } else {
+    long long before = 0;
+#pragma unroll 8
+    for (long long t = threadIdx.x; t < t0; t += UW_THREADS) before += counts[t];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    if (lane == 0) part[warp] = before;
+    __syncthreads();
+    if (warp == 0) {
+      long long sum = 0;
+#pragma unroll
+      for (int k = 0; k < UW_WARPS; k++) sum += part[k];
+      const long long own = lane < WRITE_TILES && t0 + lane < ntiles ? counts[t0 + lane] : 0;
+      long long sc = own;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const int a = __shfl_up_sync(0xffffffffu, sc, o);
+        const long long a = __shfl_up_sync(0xffffffffu, sc, o);
         if (lane >= o) sc += a;
       }
-      word_excl[q * 32 + lane] = carry + sc - cnt[q];
-      carry += __shfl_sync(0xffffffffu, sc, 31);
+      if (lane < WRITE_TILES) first[lane] = sum + sc - own;
+      if (lane == 31 && t0 + WRITE_TILES >= ntiles) *n_acc = sum + sc;
     }
+    __syncthreads();
   }
-  __syncthreads();
+#pragma unroll 1
+  for (int k = 0; k < PER_WARP; k++) {
+    const long long t = t0 + warp * PER_WARP + k;
+    if (t >= ntiles) break;
+    int own = 0;
+    unsigned w[WPL];
 #pragma unroll
-  for (int j = 0; j < UW_PER_THREAD; j++) {
-    const int q = j * UW_WARPS + warp;
-    const unsigned m = tb[q];
-    if ((m >> lane) & 1u)
-      idx_out[off + word_excl[q] + __popc(m & ((1u << lane) - 1u))] = base + j * UW_THREADS + threadIdx.x;
+    for (int q = 0; q < WPL; q++) {
+      w[q] = m[0][q];
+#pragma unroll
+      for (int kk = 1; kk < PER_WARP; kk++) w[q] = k == kk ? m[kk][q] : w[q];
+      own += __popc(w[q]);
+    }
+    int sc = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int a = __shfl_up_sync(0xffffffffu, sc, o);
+      if (lane >= o) sc += a;
+    }
+    const int total = __shfl_sync(0xffffffffu, sc, 31);
+    const long long base = t * UW_TILE;
+    long long* out = idx_out + first[warp * PER_WARP + k];
+    if (total <= UW_TILE / 8) {
+      int at = sc - own;
+#pragma unroll
+      for (int q = 0; q < WPL; q++)
+        for (unsigned b = w[q]; b; b &= b - 1) out[at++] = base + (lane * WPL + q) * 32 + __ffs(b) - 1;
+    } else {
+      for (int l = 0; l < 32; l++) {
+        int at = __shfl_sync(0xffffffffu, sc - own, l);
+#pragma unroll
+        for (int q = 0; q < WPL; q++) {
+          const unsigned b = __shfl_sync(0xffffffffu, w[q], l);
+          if (b >> lane & 1u) out[at + __popc(b & ((1u << lane) - 1u))] = base + (l * WPL + q) * 32 + lane;
+          at += __popc(b);
+        }
+      }
+    }
   }
 }
 
@@ -298,22 +279,28 @@ extern "C" int mg_unweight(const double* w_dev, const double* r_dev, int64_t n, 
   const size_t bytes = (size_t)ntiles * (sizeof(long long) + UW_WORDS * sizeof(unsigned));
   if (cudaMallocAsync(reinterpret_cast<void**>(&counts), bytes, s) != cudaSuccess) return MG_ERR_NOMEM;
   unsigned* bits = reinterpret_cast<unsigned*>(counts + ntiles);
-  const bool tma = MG_UW_TMA && (reinterpret_cast<uintptr_t>(w_dev) & 15u) == 0 &&
-                   (reinterpret_cast<uintptr_t>(r_dev) & 15u) == 0;
-  if (tma) {
-    if (cudaFuncSetAttribute(tile_count_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)UW_TMA_SMEM) != cudaSuccess) {
-      cudaFreeAsync(counts, s);
-      return MG_ERR_CUDA;
-    }
-    tile_count_tma_kernel<<<(unsigned)ntiles, UW_THREADS, UW_TMA_SMEM, s>>>(w_dev, r_dev, n, w_max, counts, bits);
-  } else {
-    tile_count_kernel<<<(unsigned)ntiles, UW_THREADS, 0, s>>>(w_dev, r_dev, n, w_max, counts, bits);
+  long long* acc = reinterpret_cast<long long*>(n_acc_dev);
+  long long* idx = reinterpret_cast<long long*>(idx_out_dev);
+  const unsigned blocks = (unsigned)((ntiles + WRITE_TILES - 1) / WRITE_TILES);
+  tile_count_kernel<<<(unsigned)ntiles, UW_THREADS, 0, s>>>(w_dev, r_dev, n, w_max, counts, bits);
+  if (ntiles > SUM_TILES) {
+    tile_scan_kernel<<<1, SCAN_T, 0, s>>>(counts, ntiles, acc);
   }
-  tile_scan_kernel<<<1, SCAN_T, 0, s>>>(counts, ntiles, reinterpret_cast<long long*>(n_acc_dev));
-  tile_write_kernel<<<(unsigned)ntiles, UW_THREADS, 0, s>>>(bits, counts, reinterpret_cast<long long*>(n_acc_dev),
-                                                            reinterpret_cast<long long*>(idx_out_dev));
-  const cudaError_t e1 = cudaGetLastError();
+  // the write pass may be set up while the pass before it drains (it waits for
+  // that pass's memory before its first read)
+  cudaLaunchAttribute early{};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(UW_THREADS);
+  cfg.stream = s;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  cudaError_t e1 = cudaLaunchKernelEx(&cfg, ntiles > SUM_TILES ? tile_write_kernel<true> : tile_write_kernel<false>,
+                                      (const unsigned*)bits, (const long long*)counts, ntiles, acc, idx);
+  const cudaError_t e3 = cudaGetLastError();
+  if (e1 == cudaSuccess) e1 = e3;
   const cudaError_t e2 = cudaFreeAsync(counts, s);
   return (e1 == cudaSuccess && e2 == cudaSuccess) ? MG_OK : MG_ERR_CUDA;
 }
