@@ -53,6 +53,29 @@ __device__ __forceinline__ R fmad(R a, R b, R c) {
   return std::fma(a, b, c);
 #endif
 }
+// (float)x and (double)f with integer instructions: the conversions run on the
+// FP64 pipe (16 cycles per warp instruction and SM), which bounds the set-up of
+// the FP32 paths.  The same results bit for bit; values outside the FP32 normal
+// range take the conversion itself.
+__device__ __forceinline__ float round_f32(double x) {
+#ifdef __CUDA_ARCH__
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x), a = hi & 0x7fffffffu;
+  uint32_t m = __funnelshift_l(lo, a, 3) - 0xC0000000u;     // exponent rebased by 896 << 23, modulo 2^32
+  m += ((lo & 0x1fffffffu) + 0x0fffffffu + (m & 1u)) >> 29;  // to nearest, ties to even
+  if (a - 0x38100000u < 0x0fd00000u) return __uint_as_float(m | (hi & 0x80000000u));  // exponents 897 .. 1149
+  if ((a | lo) == 0u) return __uint_as_float(hi);
+#endif
+  return (float)x;
+}
+__device__ __forceinline__ double widen_f64(float f) {
+#ifdef __CUDA_ARCH__
+  const uint32_t u = __float_as_uint(f), a = u & 0x7fffffffu;
+  if (a - 0x00800000u < 0x7f000000u || a == 0u)
+    return __hiloint2double((int)((a ? (a >> 3) + 0x38000000u : 0u) | (u & 0x80000000u)), (int)(u << 29));
+#endif
+  return (double)f;
+}
+
 // acc += a b, acc -= a b (complex): four fused multiply-adds
 template <typename R>
 __device__ __forceinline__ void cmac(cx<R>& acc, cx<R> a, cx<R> b) {
@@ -351,10 +374,11 @@ __device__ __forceinline__ void setup_pair(double* pairs, const double* p, int t
   pairs[t] = minus ? -d : d;
 }
 __device__ __forceinline__ double quick_inverse(double d) {
-  const float f = (float)d;
+  const float f = round_f32(d);
   const float y = 1.0f / f;
   if (!(y < 1e38f && y > -1e38f) || !(f < 1e38f && f > -1e38f)) return 1.0 / d;  // outside the FP32 range, or NaN
-  return fmad(fmad(-d, (double)y, 1.0), (double)y, (double)y);
+  const double w = widen_f64(y);
+  return fmad(fmad(-d, w, 1.0), w, w);
 }
 template <class P, class ST>
 __device__ __forceinline__ void setup_coef_pairs(const ST& st, const double* pairs, const double* kp, int c) {
@@ -385,14 +409,10 @@ __device__ __forceinline__ void setup_coef_pairs(const ST& st, const double* pai
   store_coef<float>(st, m, f, f ? (float)(r * v) : (float)r, (float)(-r * dim));
 }
 
-template <class P, typename R, typename D, class ST>
-__device__ __forceinline__ void setup_leg(const ST& st, const double* p, const double* kp, int l) {
-  using E = typename std::conditional<sizeof(R) == 4, float, D>::type;
+// external states of leg l (gluons, then t, t~) of momentum q
+template <class P, typename R, typename E, class ST>
+__device__ __forceinline__ void leg_states(const ST& st, const E (&q)[4], const double* kp, int l) {
   constexpr int N = P::N;
-  const int slot = l < 2 ? l : (l < N ? l + 2 : l - N + 2);  // gluons, then t, t~
-  E q[4];
-#pragma unroll
-  for (int mu = 0; mu < 4; mu++) q[mu] = E(p[4 * slot + mu]);
   if (l < N) {
     E b[6];
     vector_basis(q, b);
@@ -424,6 +444,16 @@ __device__ __forceinline__ void setup_leg(const ST& st, const double* p, const d
       }
     }
   }
+}
+template <class P, typename R, typename D, class ST>
+__device__ __forceinline__ void setup_leg(const ST& st, const double* p, const double* kp, int l) {
+  using E = typename std::conditional<sizeof(R) == 4, float, D>::type;
+  constexpr int N = P::N;
+  const int slot = l < 2 ? l : (l < N ? l + 2 : l - N + 2);
+  E q[4];
+#pragma unroll
+  for (int mu = 0; mu < 4; mu++) q[mu] = E(p[4 * slot + mu]);
+  leg_states<P, R, E>(st, q, kp, l);
 }
 
 // ---------------------------------------------------------------------------
@@ -574,6 +604,133 @@ __device__ __forceinline__ void vec_task(const ST& st, const RW& row) {
   g.c[2] = mul_i((u12 - u03) + (l21 - l30));
   g.c[3] = (u02 - u13) - (l20 - l31);
   st.st(row.v[2], g);
+}
+
+// ---------------------------------------------------------------------------
+// one thread per event (two gluons): the store in registers -- every index is a
+// constant once the task calls are inlined
+// ---------------------------------------------------------------------------
+template <typename R, int N, int NV>
+struct RegStore {
+  static constexpr int NSUB = 1 << N;
+  static constexpr int S_K = 0, S_PT = 4 * NSUB, S_CF = S_PT + 8, S_CG = S_CF + 2 * NSUB, NS = S_CG + NSUB;
+  mutable V4<R> v[NV];
+  mutable R sc[NS];
+  __device__ __forceinline__ V4<R> ld(int i) const { return v[i]; }
+  __device__ __forceinline__ void st(int i, const V4<R>& o) const { v[i] = o; }
+  __device__ __forceinline__ M4<R> mom(int off) const { return {{sc[off], sc[off + 1], sc[off + 2], sc[off + 3]}}; }
+  __device__ __forceinline__ M4<R> K(int mask) const { return mom(S_K + 4 * mask); }
+  __device__ __forceinline__ cx<R> cf(int mask) const { return {sc[S_CF + 2 * mask], sc[S_CF + 2 * mask + 1]}; }
+};
+
+// (p_t - K)^2 - m2 (f) or K^2 of the subset m; m and f are constants once
+// inlined.  FP64 amplitudes: compensated like inv_mass2, term by term.
+template <int N, typename R, typename D>
+__device__ __forceinline__ D subset_mass2(const D (&q)[N + 2][4], bool f, int m, D m2) {
+  constexpr bool comp = sizeof(R) == 8 && sizeof(D) == 8;
+  D hi = -m2, lo = D(0);
+#pragma unroll
+  for (int mu = 0; mu < 4; mu++) {
+    D ch = D(0), cl = D(0);
+    bool first = true;
+    if (f) {
+      ch = q[N][mu];
+      first = false;
+    }
+#pragma unroll
+    for (int i = 0; i < N; i++)
+      if (m >> i & 1) {
+        const D x = (i < 2) != f ? q[i][mu] : -q[i][mu];  // q: physical momenta, incoming first
+        if (first) {
+          ch = x;
+        } else if constexpr (comp) {
+          D e;
+          two_sum(ch, x, ch, e);
+          cl += e;
+        } else {
+          ch += x;
+        }
+        first = false;
+      }
+    if constexpr (comp) {
+      const D sq = ch * ch;
+      const D sq_lo = fmad(ch, ch, -sq) + D(2) * ch * cl;
+      D e;
+      two_sum(hi, mu == 0 ? sq : -sq, hi, e);
+      lo += mu == 0 ? e + sq_lo : e - sq_lo;
+    } else {
+      hi = fmad(mu == 0 ? ch : -ch, ch, hi);
+    }
+  }
+  return comp ? hi + lo : hi;
+}
+
+// set-up of a RegStore from the event's momenta
+template <class P, typename R, typename D, class ST>
+__device__ __forceinline__ void setup_thread(const ST& st, const double* p, const double* kp) {
+  constexpr int N = P::N;
+  D q[N + 2][4];  // gluons, top, antitop
+  R k[N + 2][4];
+#pragma unroll
+  for (int i = 0; i < N + 2; i++)
+#pragma unroll
+    for (int mu = 0; mu < 4; mu++) {
+      const double x = p[4 * (i < 2 ? i : (i < N ? i + 2 : i - N + 2)) + mu];
+      if constexpr (sizeof(D) == 8)
+        q[i][mu] = x;
+      else
+        q[i][mu] = round_f32(x);
+      if constexpr (sizeof(R) == 8)
+        k[i][mu] = x;
+      else
+        k[i][mu] = round_f32(x);
+    }
+#pragma unroll
+  for (int m = 0; m < ST::NSUB; m++)
+#pragma unroll
+    for (int mu = 0; mu < 4; mu++) {
+      R s = R(0);
+      bool first = true;
+#pragma unroll
+      for (int i = 0; i < N; i++)
+        if (m >> i & 1) {
+          const R x = i < 2 ? k[i][mu] : -k[i][mu];
+          s = first ? x : s + x;
+          first = false;
+        }
+      st.sc[ST::S_K + 4 * m + mu] = s;
+    }
+#pragma unroll
+  for (int mu = 0; mu < 4; mu++) {
+    st.sc[ST::S_PT + mu] = k[N][mu];
+    st.sc[ST::S_PT + 4 + mu] = k[N + 1][mu];
+  }
+  const D g = D(kp[0]), mt = D(kp[1]), dim = mt * D(kp[2]);
+#pragma unroll
+  for (int c = 0; c < 2 * ST::NSUB; c++) {
+    const bool f = (c >> N) != 0;
+    const int m = c & (ST::NSUB - 1);
+    if (!is_propagator<N>(c)) continue;
+    const D v = subset_mass2<N, R, D>(q, f, m, f ? mt * mt : D(0));
+    const D den = f ? fmad(v, v, dim * dim) : v;
+    D r;
+    if constexpr (sizeof(R) == 4 && sizeof(D) == 8)
+      r = -g * quick_inverse(den);
+    else
+      r = -g / den;
+    if constexpr (sizeof(R) == 4 && sizeof(D) == 8)
+      store_coef<float>(st, m, f, f ? round_f32(r * v) : round_f32(r), f ? round_f32(-r * dim) : 0.f);
+    else
+      store_coef<R>(st, m, f, f ? R(r * v) : R(r), R(-r * dim));
+  }
+  using E = typename std::conditional<sizeof(R) == 4, float, D>::type;
+#pragma unroll
+  for (int l = 0; l < N + 2; l++) {
+    E e[4];
+#pragma unroll
+    for (int mu = 0; mu < 4; mu++) e[mu] = E(k[l][mu]);
+    leg_states<P, R, E>(st, e, kp, l);
+  }
 }
 
 // x of the subset bits of the gluon helicities hg: bit i of `mask` set ->

@@ -1067,9 +1067,98 @@ def emit_uuttg(tag: str) -> str:
     L.extend(_colour_quadratic(K, 4))
     L.append("#undef JAMP")
     L.append("}")
+    L += _uuttg_thread_sum(dec)
     L.append(f"}};  // struct {tag}")
     L.append("}  // namespace mg")
     return "\n".join(L) + "\n"
+
+
+def _uuttg_thread_sum(dec) -> list[str]:
+    """Every helicity of an event by one thread: each current once per helicity
+    combination of its own legs (light-line currents per u helicity and gluon,
+    top-line ones per top, antitop and gluon), the u u~ pair with opposite
+    helicities only -- with equal ones every product has an exactly zero spinor
+    component as a factor.  The diagrams with the gluon on the light line and
+    the three-gluon diagram close on the top current, the others on the light
+    current: A = U.Hc and A = Lc.W."""
+    L = ["// sum over the helicities whose bit of `good` is set, one thread per event",
+         "template <typename R, typename D, typename A>",
+         "__device__ static __forceinline__ A thread_sum(const double* __restrict__ p, const double* __restrict__ kp,",
+         "                                               const unsigned good) {",
+         "  R ev[NSLOT];", "  prepare<R, D>(p, kp, ev, 1);",
+         "#define EV(k) ev[k]",
+         "#define ING(i) FermIngr<R>{EV(5 * (i)), EV(5 * (i) + 1), EV(5 * (i) + 2), EV(5 * (i) + 3), EV(5 * (i) + 4)}",
+         "#define MOM(k) M4<R>{{EV(k), EV((k) + 1), EV((k) + 2), EV((k) + 3)}}",
+         "  const R g = R(kp[0]), mt = R(kp[1]);",
+         "  const cx<R> ig = {R(0), g};",
+         "  const cx<R> mi_q2 = {R(0), -EV(56)}, mi_s = {R(0), -EV(57)};  // -i/q34^2, -i/s",
+         "  // light line: currents, times -i/s, of u helicity 2 h - 1 (u~ opposite); top line: times -i/q34^2",
+         "  V4<R> Lc[2], Hc[2][2];",
+         "#pragma unroll",
+         "  for (int h = 0; h < 2; h++) Lc[h] = ffv_vcur<R>(ext_vbar<R>(ING(1), 1 - 2 * h), ext_u<R>(ING(0), 2 * h - 1), mi_s * ig);",
+         "#pragma unroll",
+         "  for (int s = 0; s < 2; s++)",
+         "#pragma unroll",
+         "    for (int b = 0; b < 2; b++)",
+         "      Hc[s][b] = ffv_vcur<R>(ext_ubar<R>(ING(2), 2 * s - 1), ext_v<R>(ING(3), 2 * b - 1), mi_q2 * ig);",
+         "  const R e1[3] = {EV(20), EV(21), EV(22)}, e2[3] = {EV(23), EV(24), EV(25)};",
+         "  const M4<R> kx = MOM(42), ky = MOM(46);",
+         "  M4<R> ka, kb, kd;  // 2 ky + kx, 2 kx + ky, kx - ky",
+         "  for (int mu = 0; mu < 4; mu++) {",
+         "    ka.v[mu] = R(2) * ky[mu] + kx[mu];",
+         "    kb.v[mu] = R(2) * kx[mu] + ky[mu];",
+         "    kd.v[mu] = kx[mu] - ky[mu];",
+         "  }",
+         "  A acc = A(0);",
+         "#pragma unroll 1",
+         "  for (int e = 0; e < 2; e++) {  // gluon helicity 2 e - 1",
+         "    const V4<R> eps = ext_vector<R>(e1, e2, R(2 * e - 1), true);",
+         "    V4<R> U[2][3];  // gluon off the u end, off the u~ end, three-gluon vertex",
+         "#pragma unroll",
+         "    for (int h = 0; h < 2; h++) {",
+         "      const Sp<R> w0 = ext_u<R>(ING(0), 2 * h - 1), w1 = ext_vbar<R>(ING(1), 1 - 2 * h);",
+         "      U[h][0] = ffv_vcur<R>(w1, ffv_col<R>(eps, w0, MOM(26), R(0), cx<R>{EV(50), R(0)}), ig);",
+         "      U[h][1] = ffv_vcur<R>(ffv_row<R>(w1, eps, MOM(30), R(0), cx<R>{EV(51), R(0)}), w0, ig);",
+         "      const cx<R> de = g * dot(kd, eps), al = g * dot(ka, Lc[h]), le = g * dot(Lc[h], eps);",
+         "      for (int mu = 0; mu < 4; mu++)",
+         "        U[h][2].c[mu] = de * Lc[h].c[mu] + al * eps.c[mu] - kb[mu] * le;",
+         "    }",
+         "    Sp<R> sD[2];",
+         "#pragma unroll",
+         "    for (int b = 0; b < 2; b++)",
+         "      sD[b] = ffv_col<R>(eps, ext_v<R>(ING(3), 2 * b - 1), MOM(38), mt, cx<R>{EV(54), EV(55)});",
+         "#pragma unroll",
+         "    for (int s = 0; s < 2; s++) {",
+         "      const Sp<R> w2 = ext_ubar<R>(ING(2), 2 * s - 1);",
+         "      const Sp<R> sC = ffv_row<R>(w2, eps, MOM(34), mt, cx<R>{EV(52), EV(53)});",
+         "#pragma unroll",
+         "      for (int b = 0; b < 2; b++) {",
+         "        const V4<R> vC = ffv_vcur<R>(sC, ext_v<R>(ING(3), 2 * b - 1), ig);",
+         "        const V4<R> vD = ffv_vcur<R>(w2, sD[b], ig);",
+         "#pragma unroll",
+         "        for (int h = 0; h < 2; h++) {",
+         "          const cx<R> a[5] = {dot(U[h][0], Hc[s][b]), dot(U[h][1], Hc[s][b]), dot(Lc[h], vC), dot(Lc[h], vD),",
+         "                              dot(U[h][2], Hc[s][b])};",
+         "          cx<R> jamp[NCOL];"]
+    for m in range(4):
+        terms = []
+        for d in range(5):
+            re, im = dec[d][m]
+            if re == 0 and im == 0:
+                continue
+            if im == 0:
+                terms.append(f"R({float(re)!r}) * a[{d}]")
+            elif re == 0:
+                terms.append(f"R({float(im)!r}) * mul_i(a[{d}])")
+            else:
+                terms.append(f"cx<R>{{R({float(re)!r}), R({float(im)!r})}} * a[{d}]")
+        L.append(f"          jamp[{m}] = " + " + ".join(terms) + ";")
+    L += ["          const R v = colour_quadratic<R>(jamp, 1);",
+          "          const int hel = (h << 4) | ((1 - h) << 3) | (s << 2) | (b << 1) | e;",
+          "          if (good >> hel & 1u) acc += (A)v;",
+          "        }", "      }", "    }", "  }", "  return acc;",
+          "#undef MOM", "#undef ING", "#undef EV", "}"]
+    return L
 
 
 # processes emitted as straight-line code cut into separately compiled chunk
@@ -1190,11 +1279,11 @@ VERTEX_CALLS = {"f32": {"ggttgg", "ggttggg"}, "f64": set()}
 # the arithmetic of the amplitudes.  FP32 covers MG_MIXED and MG_FLOAT, FP64
 # every other mode; the helicity and colour choice of the FP32 modes keeps the
 # per-helicity program, whose choices must not move with the rounding of the
-# flows.  gg -> t t~ in FP32 keeps it too: sixteen short helicities of one
-# thread per event beat the recursion's small stages (524288 events 0.20
-# against 0.58 ms; FP64, bound by the FP64 pipe, 1.17 against 0.69 ms per 65536).
-RECURSION = {"f32": {"ggttg", "ggttgg", "ggttggg"}, "f64": {"ggtt", "ggttg", "ggttgg", "ggttggg"}}
-# of these, the mixed mode writes the flows to a workspace and contracts colour
+# flows.
+RECURSION = {"f32": {"ggtt", "ggttg", "ggttgg", "ggttggg"}, "f64": {"ggtt", "ggttg", "ggttgg", "ggttggg"}}
+# of these, |M|^2 by one thread per event that runs all helicities in registers
+THREAD_SUM = {"ggtt", "uuttg"}
+# the mixed mode writes the flows to a workspace and contracts colour
 # on the tensor cores in a second kernel (120 flows)
 RECURSION_ROWS = {"ggttggg"}
 
@@ -1221,9 +1310,15 @@ def emit_tu(proc: str, prec: str) -> tuple[str, str]:
         if rec:
             mixed = f"launch_rec_rows<{tag}_rec>(a)" if rows else f"launch_rec<{tag}_rec, float, double, double>(a)"
             flt = f"launch_rec<{tag}_rec, float, float, float>(a)"
+            if tag in THREAD_SUM:
+                mixed = f"launch_sigma_thread<{tag}_rec, float, double, double, 128, 3>(a)"
+                flt = f"launch_sigma_thread<{tag}_rec, float, float, float, 128, 3>(a)"
         else:
             mixed = f"launch_sigma<{tag}, float, {nt32}>(a)"
             flt = f"launch_sigma<{tag}, float, {nt32}, float, float>(a)"
+            if tag in THREAD_SUM:
+                mixed = f"launch_sigma_thread<{tag}, float, double, double, 128, 2>(a)"
+                flt = f"launch_sigma_thread<{tag}, float, float, float, 128, 2>(a)"
         src = f"""{head}#include "../mg_kernels.cuh"
 {inc}{prog}
 namespace mg {{
@@ -1236,8 +1331,11 @@ int sigma_{tag}_float(const LaunchArgs& a) {{ return {flt}; }}
     if rec:
         fp64, hel, sel, paper = (f"launch_rec<{tag}_rec, double, double, double, {m}>(a)"
                                  for m in ("REC_SIGMA", "REC_HELICITIES", "REC_SELECT", "REC_PAPER"))
+        if tag in THREAD_SUM:
+            fp64 = f"launch_sigma_thread<{tag}_rec, double, double, double, 128, 1>(a)"
     else:
-        fp64, hel, sel, paper = (f"launch_sigma<{tag}, double, {nt64}>(a)", f"launch_helicities<{tag}, {nt64}>(a)",
+        fp64, hel, sel, paper = ((f"launch_sigma_thread<{tag}, double, double, double, 128, 1>(a)" if tag in THREAD_SUM
+                                  else f"launch_sigma<{tag}, double, {nt64}>(a)"), f"launch_helicities<{tag}, {nt64}>(a)",
                                  f"launch_select<{tag}, double, {nt64}>(a)", f"launch_sigma_paper<{tag}, {nt64}>(a)")
     ncol = FIXED_NCOL.get(tag) or math.factorial(n)
     tck = ((ncol + 15) // 16) * 16 if rows else 0

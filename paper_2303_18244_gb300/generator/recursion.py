@@ -81,6 +81,7 @@ class Recursion:
         self.items: dict = {}      # key -> (gluons sorted, spin bits)
         self.tasks: dict = {}      # stage name -> list of items to compute
         self.base: dict = {}
+        self._lev: dict = {}
         self._collect()
         self._layout()
 
@@ -322,26 +323,27 @@ class Recursion:
             self._lev[key] = 1 + max([self.level(k) for k in self.deps(key)], default=-1)
         return self._lev[key]
 
+    def routine(self, key) -> str:
+        """The task call of an item ({row}: its table line)."""
+        kind, m = key[0], len(key[1])
+        if kind == "J":
+            return f"j_task<{m}, R>(st, {{row}}, kp)" if m < 3 or key[1][0] == min(key[1]) else "comb_task<R>(st, {row})"
+        if kind in "RC":
+            return f"line_task<{m}, R>(st, {{row}}, kp)"
+        if kind == "A":
+            return f"amp_task<{m}, R>(st, {{row}})"
+        if kind == "S":
+            return "amp_task<1, R>(st, {row}, S0<R>)" if self.n == 4 else "amp_task<1, R>(st, {row})"
+        return "vec_task<R>(st, {row})"
+
     def stages(self):
         """[(level, routine, row width, rows)]: task lists in dependency order;
         lists of one level are independent of each other."""
-        self._lev: dict = {}
         lists: dict = {}
         for stage, keys in self.tasks.items():
             for key in keys:
                 lev = 99 if self.late(key) else self.level(key)
-                if stage[0] == "J":
-                    fn = f"j_task<{len(key[1])}, R>(st, {{row}}, kp)"
-                elif stage[0] == "K":
-                    fn = "comb_task<R>(st, {row})"
-                elif stage[0] in "RC":
-                    fn = f"line_task<{len(key[1])}, R>(st, {{row}}, kp)"
-                elif stage[0] == "A":
-                    fn = f"amp_task<{len(key[1])}, R>(st, {{row}})"
-                elif stage[0] == "S":
-                    fn = "amp_task<1, R>(st, {row}, S0<R>)" if self.n == 4 else "amp_task<1, R>(st, {row})"
-                else:
-                    fn = "vec_task<R>(st, {row})"
+                fn = "rec::" + self.routine(key)
                 lists.setdefault((lev, fn), []).extend(self.table(stage, [key]))
         return sorted([(lev, fn, rows) for (lev, fn), rows in lists.items()], key=lambda x: x[0])
 
@@ -565,6 +567,42 @@ def flow_order(n: int) -> list[tuple]:
     return sorted(words(n), key=lambda w: (w[-1:] + w) if n > 4 else w)
 
 
+def _thread_sum(rec: Recursion) -> list[str]:
+    """Two gluons: every helicity of an event by one thread, straight line in
+    registers, the antitop spins one after the other (the columns and closing
+    vectors of one spin at a time)."""
+    L = ["  // sum over the helicities whose bit of `good` is set, one thread per event",
+         "  template <typename R, typename D, typename A>",
+         "  __device__ static __forceinline__ A thread_sum(const double* p, const double* kp, const unsigned good) {",
+         "    using namespace rec;",
+         f"    const RegStore<R, {rec.n}, {rec.nvec}> st{{}};",
+         "    setup_thread<" + "P_SELF" + ", R, D>(st, p, kp);", "    A acc = A(0);"]
+    calls: dict = {None: [], 0: [], 1: []}
+    for stage, keys in rec.tasks.items():
+        for key in keys:
+            rows = rec.table(stage, [key])
+            for row, (hel, s, b) in zip(rows, rec._combos(key)):
+                w = ((len(row) + 7) // 8) * 8
+                lit = f"Row<{w}>{{{{" + ", ".join(str(x) for x in row + [0] * (w - len(row))) + "}}"
+                when = b if key[0] in "CV" else None
+                calls[when].append((rec.level(key), rec.routine(key).format(row=lit)))
+    L += ["    " + c + ";" for _, c in sorted(calls[None], key=lambda x: x[0])]
+    for b in range(2):
+        L += ["    " + c + ";" for _, c in sorted(calls[b], key=lambda x: x[0])]
+        for s in range(2):
+            for hg in range(1 << rec.n):
+                L.append(f"    {{ cx<R> a[1][2]; flows_open<R, 1>(st, {hg}, {s}, {b}, a); flows_block<R, 1>(st, {hg}, {s}, {b}, a);")
+                L.append("      const R v = colour_form<R>(a[0]);")
+                L.append(f"      if (good >> helicity({hg}, {s}, {b}) & 1u) acc += widen<A>(v); }}")
+    L += ["    return acc;", "  }",
+          "  template <typename A>",
+          "  __device__ static __forceinline__ A widen(float v) {",
+          "    if constexpr (sizeof(A) == 8) return rec::widen_f64(v); else return v;", "  }",
+          "  template <typename A>",
+          "  __device__ static __forceinline__ A widen(double v) { return (A)v; }"]
+    return L
+
+
 def _grouped_flows(rec: Recursion, head, tag, late) -> list[str]:
     """Five gluons: 120 flows do not fit in registers, so they are closed in
     five groups by their last gluon e, all by the same code (a loop over e; the
@@ -713,12 +751,12 @@ def emit_recursion(n: int, tag: str) -> str:
                  + ", ".join("{{" + ", ".join(str(x) for x in flat[i:i + w]) + "}}" for i in range(0, len(flat), w))
                  + "};")
         if lev == 99:
-            late.append(f"    MG_REC_LOOP for (int t = tid; t < {len(rows)}; t += nt) rec::{fn.format(row=f'{name}[t]')};")
+            late.append(f"    MG_REC_LOOP for (int t = tid; t < {len(rows)}; t += nt) {fn.format(row=f'{name}[t]')};")
             continue
         if prev is not None and lev != prev:
             body.append("    sync();")
         prev = lev
-        body.append(f"    MG_REC_LOOP for (int t = tid; t < {len(rows)}; t += nt) rec::{fn.format(row=f'{name}[t]')};")
+        body.append(f"    MG_REC_LOOP for (int t = tid; t < {len(rows)}; t += nt) {fn.format(row=f'{name}[t]')};")
     L = [f"// generated by paper_2303_18244_gb300.generator for 'g g > t t~{' g' * (n - 2)}':",
          "// helicity-shared colour-ordered recursion", "#pragma once", '#include "mg_recursion.cuh"', "namespace mg {"]
     L += T
@@ -777,6 +815,8 @@ def emit_recursion(n: int, tag: str) -> str:
     else:
         L += _grouped_flows(rec, L, tag, late)
     # colour form
+    if n == 2:
+        L += [x.replace("P_SELF", f"{tag}_rec") for x in _thread_sum(rec)]
     if n > 4:
         L += _colour_form_looped(L, tag, n, K, ws)
         L += ["};", "}  // namespace mg"]

@@ -108,3 +108,64 @@ def test_flows_of_every_helicity(proc, sqrts, nevt, tmp_path):
         assert np.max(r[e, :, 1]) <= 1e-11
         tot = r[e, :, 3].sum()
         assert np.max(np.abs(r[e, :, 2] - r[e, :, 3])) <= 1e-11 * tot
+
+
+THREAD_PROGRAM = PROGRAM[:PROGRAM.index('#include "TAG.cuh"')] + r"""
+#include "TAG.cuh"
+REC
+using namespace mg;
+int main() {
+  double kp[8];
+  for (double& x : kp)
+    if (scanf("%lf", &x) != 1) return 1;
+  int nevt;
+  if (scanf("%d", &nevt) != 1) return 1;
+  for (int e = 0; e < nevt; e++) {
+    double p[TAG::NPAR * 4];
+    for (double& x : p)
+      if (scanf("%lf", &x) != 1) return 1;
+    unsigned good;
+    if (scanf("%u", &good) != 1) return 1;
+    double slab[TAG::NSLOT], want = 0.0;
+    TAG::prepare<double, double>(p, kp, slab, 1);
+    for (int h = 0; h < TAG::NHEL; h++)
+      if (good >> h & 1u) {
+        cx<double> jamp[TAG::NCOL];
+        TAG::amplitudes<double>(slab, 1, h, kp, jamp, 1);
+        want += TAG::colour_quadratic<double>(jamp, 1);
+      }
+    printf("%.17g %.17g\n", THREAD::thread_sum<double, double, double>(p, kp, good), want);
+  }
+  return 0;
+}
+"""
+
+
+@pytest.mark.parametrize("proc,sqrts,rec", [("g g > t t~", 1000.0, True), ("u u~ > t t~ g", 1200.0, False)],
+                         ids=["ggtt", "uuttg"])
+def test_thread_sum_over_helicity_lists(proc, sqrts, rec, tmp_path):
+    """One thread's sum over all helicities, for the full list, single
+    helicities and random lists, against the per-helicity program summed over
+    the same list (1e-12: the sum of a list can be a small part of its
+    helicities' currents, each within 1e-14 or so of the program's)."""
+    tag, n = emit.PROCESSES[proc]
+    (tmp_path / f"{tag}.cuh").write_text(emit.emit(proc, "f64")[1])
+    src = THREAD_PROGRAM.replace("REC", f'#include "{tag}_rec.cuh"' if rec else "")
+    if rec:
+        (tmp_path / f"{tag}_rec.cuh").write_text(recursion.emit_recursion(n, tag))
+    (tmp_path / "main.cpp").write_text(src.replace("THREAD", f"{tag}_rec" if rec else tag).replace("TAG", tag))
+    exe = tmp_path / "main"
+    subprocess.run(["g++", "-O0", "-std=c++17", f"-I{tmp_path}", f"-I{CSRC}", "-o", str(exe), str(tmp_path / "main.cpp")],
+                   check=True)
+    nhel = 1 << len(proc.replace(">", " ").split())
+    rng = np.random.default_rng(3)
+    lists = [(1 << nhel) - 1] + [1 << h for h in range(nhel)] + [int(rng.integers(1, 1 << nhel)) for _ in range(10)]
+    p = process_momenta(proc, sqrts, len(lists), 58)
+    lines = [" ".join(repr(float(x)) for x in _couplings(proc)), str(len(lists))]
+    lines += [" ".join(repr(float(x)) for x in ev.ravel()) + f" {m}" for ev, m in zip(p, lists)]
+    out = subprocess.run([str(exe)], input="\n".join(lines) + "\n", capture_output=True, text=True, check=True).stdout
+    r = np.array([[float(x) for x in ln.split()] for ln in out.splitlines()])
+    assert r.shape == (len(lists), 2) and np.all(r[0] > 0)
+    zero = r[:, 1] == 0.0  # equal u and u~ helicities: exactly zero on both sides
+    assert np.all(r[zero, 0] == 0.0)
+    assert np.max(np.abs(r[~zero, 0] / r[~zero, 1] - 1)) <= 1e-12
