@@ -102,83 +102,68 @@ __host__ __device__ constexpr uint32_t tile_off(int row, int k, int K) {
 
 }  // namespace tc
 
-// The per-helicity colour form of a CTA of 128 events, shared by the fused
-// kernels.  (1) Each event's thread writes its flows, scaled by a power of two
-// s = 2^-ex that puts max |J| in [1, 2), as FP16 hi + lo into the four operand
-// tiles (re_hi, re_lo, im_hi, im_lo; row = event); returns s.
+// The colour form of 128 rows (TMEM lane = row), Re and Im one after the other
+// through one pair of operand tiles.  (1) Each row's thread writes its part's
+// flows, scaled by the row's power of two s, as FP16 hi + lo.
 template <class P, int K>
-__device__ __forceinline__ float colour_operands(unsigned char* atile, size_t a_tile, int row,
-                                                 const float (&fr)[P::NCOL], const float (&fi)[P::NCOL]) {
+__device__ __forceinline__ float colour_scale(const float (&fr)[P::NCOL], const float (&fi)[P::NCOL]) {
   float mx = 0.f;
 #pragma unroll
   for (int k = 0; k < P::NCOL; k++) mx = fmaxf(mx, fmaxf(fabsf(fr[k]), fabsf(fi[k])));
   const int ex = mx > 0.f ? ((int)((__float_as_uint(mx) >> 23) & 0xff) - 127) : 0;
-  const float s = __uint_as_float((uint32_t)(127 - ex) << 23);  // 2^-ex
+  return __uint_as_float((uint32_t)(127 - ex) << 23);  // 2^-ex: max |J| in [1, 2)
+}
+template <class P, int K>
+__device__ __forceinline__ void colour_operands(unsigned char* atile, size_t a_tile, int row, float s,
+                                                const float (&f)[P::NCOL]) {
 #pragma unroll
   for (int j = 0; j < K / 8; j++) {
-    __align__(16) __half hr[8], lr[8], hi_[8], li[8];
+    __align__(16) __half hi[8], lo[8];
 #pragma unroll
     for (int q = 0; q < 8; q++) {
       const int k = 8 * j + q;
-      const float xr = k < P::NCOL ? s * fr[k < P::NCOL ? k : 0] : 0.f;
-      const float xi = k < P::NCOL ? s * fi[k < P::NCOL ? k : 0] : 0.f;
-      hr[q] = __float2half_rn(xr);
-      lr[q] = __float2half_rn(xr - __half2float(hr[q]));
-      hi_[q] = __float2half_rn(xi);
-      li[q] = __float2half_rn(xi - __half2float(hi_[q]));
+      const float x = k < P::NCOL ? s * f[k < P::NCOL ? k : 0] : 0.f;
+      hi[q] = __float2half_rn(x);
+      lo[q] = __float2half_rn(x - __half2float(hi[q]));
     }
     const uint32_t off = tc::tile_off(row, 8 * j, K);
-    *reinterpret_cast<uint4*>(atile + 0 * a_tile + off) = *reinterpret_cast<const uint4*>(hr);
-    *reinterpret_cast<uint4*>(atile + 1 * a_tile + off) = *reinterpret_cast<const uint4*>(lr);
-    *reinterpret_cast<uint4*>(atile + 2 * a_tile + off) = *reinterpret_cast<const uint4*>(hi_);
-    *reinterpret_cast<uint4*>(atile + 3 * a_tile + off) = *reinterpret_cast<const uint4*>(li);
+    *reinterpret_cast<uint4*>(atile + off) = *reinterpret_cast<const uint4*>(hi);
+    *reinterpret_cast<uint4*>(atile + a_tile + off) = *reinterpret_cast<const uint4*>(lo);
   }
-  return s;
 }
 
-// (2) One elected thread: D_re = (A_re_hi + A_re_lo) . KNUM into TMEM columns
-// [0, N), D_im likewise into [N, 2N); completion arrives on mma_bar.
+// (2) One elected thread: D = (A_hi + A_lo) . KNUM into the N columns at d;
+// completion arrives on mma_bar.
 template <int K, int N>
-__device__ __forceinline__ void colour_mma(uint32_t tmem, uint32_t a_addr, uint32_t b_addr, size_t a_tile,
+__device__ __forceinline__ void colour_mma(uint32_t d, uint32_t a_addr, uint32_t b_addr, size_t a_tile,
                                            uint64_t* mma_bar) {
   constexpr uint32_t idesc = tc::idesc_f16(128, N);
   constexpr uint32_t SBO = (K / 8) * 128;
   tc::fence_after_sync();
-  for (int part = 0; part < 2; part++) {  // 0: Re -> columns [0, N), 1: Im -> [N, 2N)
-    const uint32_t d = tmem + part * N;
-    for (int kk = 0; kk < K / 16; kk++) {
-      const uint64_t bd = tc::smem_desc(b_addr + kk * 2 * tc::LBO, tc::LBO, SBO);
-      const uint32_t hi_base = a_addr + (2 * part) * (uint32_t)a_tile + kk * 2 * tc::LBO;
-      const uint32_t lo_base = a_addr + (2 * part + 1) * (uint32_t)a_tile + kk * 2 * tc::LBO;
-      tc::mma_f16(d, tc::smem_desc(hi_base, tc::LBO, SBO), bd, idesc, kk > 0 ? 1u : 0u);
-      tc::mma_f16(d, tc::smem_desc(lo_base, tc::LBO, SBO), bd, idesc, 1u);
-    }
+  for (int kk = 0; kk < K / 16; kk++) {
+    const uint64_t bd = tc::smem_desc(b_addr + kk * 2 * tc::LBO, tc::LBO, SBO);
+    const uint32_t at = a_addr + kk * 2 * tc::LBO;
+    tc::mma_f16(d, tc::smem_desc(at, tc::LBO, SBO), bd, idesc, kk > 0 ? 1u : 0u);
+    tc::mma_f16(d, tc::smem_desc(at + (uint32_t)a_tile, tc::LBO, SBO), bd, idesc, 1u);
   }
   tc::mma_commit(mma_bar);
 }
 
-// (3) Warp-collective: the event's row of D read from its TMEM lane and
-// contracted with its flows, sum_k Re J_k D_re,k + Im J_k D_im,k (still
-// scaled by s).
+// (3) Warp-collective: the row of D at TMEM address d contracted with the
+// flows, sum_k J_k D_k (still scaled by s).
 template <class P, int N>
-__device__ __forceinline__ float colour_readback(uint32_t lane_base, const float (&fr)[P::NCOL],
-                                                 const float (&fi)[P::NCOL]) {
-  float dsum = 0.f;
+__device__ __forceinline__ float colour_readback(uint32_t d, const float (&f)[P::NCOL]) {
+  float sum = 0.f;
 #pragma unroll
   for (int c = 0; c < N; c += 16) {
-    float dr[16], di[16];
-    tc::tmem_ld16(lane_base + c, dr);
-    tc::tmem_ld16(lane_base + N + c, di);
+    float v[16];
+    tc::tmem_ld16(d + c, v);
     tc::tmem_wait_ld();
 #pragma unroll
-    for (int q = 0; q < 16; q++) {
-      if (c + q < P::NCOL) {
-        dsum = fmaf(fr[c + q < P::NCOL ? c + q : 0], dr[q], dsum);
-        dsum = fmaf(fi[c + q < P::NCOL ? c + q : 0], di[q], dsum);
-      }
-    }
+    for (int q = 0; q < 16; q++)
+      if (c + q < P::NCOL) sum = fmaf(f[c + q < P::NCOL ? c + q : 0], v[q], sum);
   }
-  return dsum;
+  return sum;
 }
 
 // FP16 bit pattern of an integer, or -1 if it is not exactly representable.
@@ -220,7 +205,7 @@ struct LayoutRows {
   static constexpr size_t a_tile = size_t(128) * K * 2;  // FP16 [128][K]
   static constexpr size_t b_tile = size_t(N) * K * 2;    // FP16 [N][K]
   static constexpr size_t a_off = 128;                    // MMA bar, TMEM address
-  static constexpr size_t b_off = a_off + 4 * a_tile;
+  static constexpr size_t b_off = a_off + 2 * a_tile;   // one part (Re or Im) at a time: hi, lo
   static constexpr size_t base_bytes = b_off + b_tile;
   static constexpr uint32_t tmem_cols = (2 * N <= 32) ? 32 : (2 * N <= 64) ? 64 : (2 * N <= 128) ? 128 : 256;
 };

@@ -76,6 +76,14 @@ __device__ __forceinline__ double widen_f64(float f) {
   return (double)f;
 }
 
+template <typename T>
+__device__ __forceinline__ T narrow(double x) {
+  if constexpr (sizeof(T) == 4)
+    return round_f32(x);
+  else
+    return x;
+}
+
 // acc += a b, acc -= a b (complex): four fused multiply-adds
 template <typename R>
 __device__ __forceinline__ void cmac(cx<R>& acc, cx<R> a, cx<R> b) {
@@ -186,7 +194,8 @@ struct Store {
   static constexpr int NS = S_CG + NSUB;
   static constexpr size_t vec_bytes = size_t(NV) * 8 * sizeof(R);
   static constexpr size_t pair_off = vec_bytes + size_t(NS) * sizeof(R);  // setup_pair (FP32)
-  static constexpr size_t bytes = pair_off + (sizeof(R) == 4 ? size_t((N + 1) * (N + 2) / 2) * sizeof(double) : 0);
+  static constexpr size_t mom_off = pair_off + (sizeof(R) == 4 ? size_t((N + 1) * (N + 2) / 2) * sizeof(double) : 0);
+  static constexpr size_t bytes = mom_off + size_t(N + 2) * 4 * sizeof(R);  // the event's momenta in R
   Pack<R>* p;
   R* sc;
   __device__ __forceinline__ explicit Store(void* mem)
@@ -194,6 +203,9 @@ struct Store {
         sc(reinterpret_cast<R*>(reinterpret_cast<unsigned char*>(mem) + vec_bytes)) {}
   __device__ __forceinline__ double* pairs() const {
     return reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(p) + pair_off);
+  }
+  __device__ __forceinline__ R* momenta() const {
+    return reinterpret_cast<R*>(reinterpret_cast<unsigned char*>(p) + mom_off);
   }
   __device__ __forceinline__ V4<R> ld(int v) const {
     V4<R> o;
@@ -278,27 +290,27 @@ __device__ __forceinline__ D inv_mass2_masked(const double* p, const int (&slot)
   }
 }
 
-// Tasks of the set-up, in three lists that a thread group strides over:
-//   subset m in [0, 2^N): momentum sum; fermion denominators of the proper
-//   subsets; gluon denominators of two or more gluons
-//   leg l in [0, N + 2): external wavefunctions.
-// g is folded into the row of the outgoing top (one factor per amplitude).
-template <class P, typename R, typename D, class ST>
-__device__ __forceinline__ void setup_momenta(const ST& st, const double* p, int m) {
+// Tasks of the set-up, in lists that a thread group strides over, after the
+// momenta have been brought to R (k[NPAR][4]): subset m in [0, 2^N): momentum
+// sum; denominators of the propagators' subsets; leg l in [0, N + 2): external
+// wavefunctions.  kr: g_s, m_t in R.  g is folded into the row of the outgoing
+// top (one factor per amplitude).
+template <class P, typename R, class ST>
+__device__ __forceinline__ void setup_momenta(const ST& st, const R* k, int m) {
   constexpr int N = P::N;
-  R k[4] = {R(0), R(0), R(0), R(0)};
+  R t[4] = {R(0), R(0), R(0), R(0)};
 #pragma unroll
   for (int i = 0; i < N; i++) {
     const int slot = i < 2 ? i : i + 2;
     const R sg = !(m >> i & 1) ? R(0) : (i < 2 ? R(1) : R(-1));
 #pragma unroll
-    for (int mu = 0; mu < 4; mu++) k[mu] = k[mu] + sg * R(p[4 * slot + mu]);
+    for (int mu = 0; mu < 4; mu++) t[mu] = fmad(sg, k[4 * slot + mu], t[mu]);
   }
 #pragma unroll
-  for (int mu = 0; mu < 4; mu++) st.sc[ST::S_K + 4 * m + mu] = k[mu];
+  for (int mu = 0; mu < 4; mu++) st.sc[ST::S_K + 4 * m + mu] = t[mu];
   if (m < 2) {
 #pragma unroll
-    for (int mu = 0; mu < 4; mu++) st.sc[ST::S_PT + 4 * m + mu] = R(p[8 + 4 * m + mu]);
+    for (int mu = 0; mu < 4; mu++) st.sc[ST::S_PT + 4 * m + mu] = k[8 + 4 * m + mu];
   }
 }
 // c in [0, 2^(N+1)): bit N selects the fermion denominators
@@ -406,12 +418,12 @@ __device__ __forceinline__ void setup_coef_pairs(const ST& st, const double* pai
   }
   const double dim = mt * wt;
   const double r = -g * quick_inverse(f ? fmad(v, v, dim * dim) : v);
-  store_coef<float>(st, m, f, f ? (float)(r * v) : (float)r, (float)(-r * dim));
+  store_coef<float>(st, m, f, round_f32(f ? r * v : r), f ? round_f32(-r * dim) : 0.f);
 }
 
 // external states of leg l (gluons, then t, t~) of momentum q
 template <class P, typename R, typename E, class ST>
-__device__ __forceinline__ void leg_states(const ST& st, const E (&q)[4], const double* kp, int l) {
+__device__ __forceinline__ void leg_states(const ST& st, const E (&q)[4], const R* kr, int l) {
   constexpr int N = P::N;
   if (l < N) {
     E b[6];
@@ -422,9 +434,9 @@ __device__ __forceinline__ void leg_states(const ST& st, const E (&q)[4], const 
     st.st(base + 1, ext_vector<R>(e1, e2, R(1), l >= 2));
   } else {
     E f[5];
-    fermion_ingredients(q, E(kp[1]), f);
+    fermion_ingredients(q, E(kr[1]), f);
     const FermIngr<R> fi = {R(f[0]), R(f[1]), R(f[2]), R(f[3]), R(f[4])};
-    const R g = R(kp[0]);
+    const R g = kr[0];
 #pragma unroll
     for (int h = 0; h < 2; h++) {
       const int lam = 2 * h - 1;
@@ -445,19 +457,16 @@ __device__ __forceinline__ void leg_states(const ST& st, const E (&q)[4], const 
     }
   }
 }
-template <class P, typename R, typename D, class ST>
-__device__ __forceinline__ void setup_leg(const ST& st, const double* p, const double* kp, int l) {
-  using E = typename std::conditional<sizeof(R) == 4, float, D>::type;
+template <class P, typename R, class ST>
+__device__ __forceinline__ void setup_leg(const ST& st, const R* k, const R* kr, int l) {
   constexpr int N = P::N;
   const int slot = l < 2 ? l : (l < N ? l + 2 : l - N + 2);
-  E q[4];
-#pragma unroll
-  for (int mu = 0; mu < 4; mu++) q[mu] = E(p[4 * slot + mu]);
-  leg_states<P, R, E>(st, q, kp, l);
+  const R q[4] = {k[4 * slot], k[4 * slot + 1], k[4 * slot + 2], k[4 * slot + 3]};
+  leg_states<P, R, R>(st, q, kr, l);
 }
 
 // ---------------------------------------------------------------------------
-// tasks; row: the task's line of the stage table
+// tasks; row: the task's line of the stage table; kr: g_s, m_t in R
 // ---------------------------------------------------------------------------
 template <int W>
 struct alignas(16) Row {
@@ -473,7 +482,7 @@ struct alignas(16) Row {
 // the two masks of every split, the mask of w, the destination (and for
 // pairs the destination of J(w reversed) = -J(w)).
 template <int M, typename R, class ST, class RW>
-__device__ __forceinline__ void j_task(const ST& st, const RW& row, const double* kp) {
+__device__ __forceinline__ void j_task(const ST& st, const RW& row, const R* kr) {
   constexpr int NSUBW = M * (M + 1) / 2 - 1;
   // position of the sub-current [i, j) in the table
   auto at = [](int i, int j) constexpr {
@@ -513,7 +522,7 @@ __device__ __forceinline__ void j_task(const ST& st, const RW& row, const double
     }
   }
   if constexpr (M > 2) {
-    const R g = R(kp[0]);
+    const R g = kr[0];
 #pragma unroll
     for (int i = 1; i < M - 1; i++)
 #pragma unroll
@@ -576,7 +585,7 @@ __device__ __forceinline__ void amp_task(const ST& st, const RW& row, int dst0 =
 // full line; table: the pairs, destination, line (0 top, 1 antitop), mask of
 // the momenta it absorbed, mask of the denominator
 template <int NT, typename R, class ST, class RW>
-__device__ __forceinline__ void line_task(const ST& st, const RW& row, const double* kp) {
+__device__ __forceinline__ void line_task(const ST& st, const RW& row, const R* kr) {
   const V4<R> t = line_sum<NT, R>(st, row);
   const int line = row.v[2 * NT + 1];
   const M4<R> e = st.mom(ST::S_PT + 4 * line), k = st.K(row.v[2 * NT + 2]);
@@ -586,7 +595,7 @@ __device__ __forceinline__ void line_task(const ST& st, const RW& row, const dou
   M4<R> Q;
 #pragma unroll
   for (int mu = 0; mu < 4; mu++) Q.v[mu] = e.v[mu] - k.v[mu];
-  st.st(row.v[2 * NT], row_prop(t, Q, R(kp[1]), c));
+  st.st(row.v[2 * NT], row_prop(t, Q, kr[1], c));
 }
 // V with V.J = row Jslash column; table: row, column, destination
 template <typename R, class ST, class RW>
@@ -667,7 +676,7 @@ __device__ __forceinline__ D subset_mass2(const D (&q)[N + 2][4], bool f, int m,
 
 // set-up of a RegStore from the event's momenta
 template <class P, typename R, typename D, class ST>
-__device__ __forceinline__ void setup_thread(const ST& st, const double* p, const double* kp) {
+__device__ __forceinline__ void setup_thread(const ST& st, const double* p, const double* kp, const R* kr) {
   constexpr int N = P::N;
   D q[N + 2][4];  // gluons, top, antitop
   R k[N + 2][4];
@@ -676,14 +685,8 @@ __device__ __forceinline__ void setup_thread(const ST& st, const double* p, cons
 #pragma unroll
     for (int mu = 0; mu < 4; mu++) {
       const double x = p[4 * (i < 2 ? i : (i < N ? i + 2 : i - N + 2)) + mu];
-      if constexpr (sizeof(D) == 8)
-        q[i][mu] = x;
-      else
-        q[i][mu] = round_f32(x);
-      if constexpr (sizeof(R) == 8)
-        k[i][mu] = x;
-      else
-        k[i][mu] = round_f32(x);
+      q[i][mu] = narrow<D>(x);
+      k[i][mu] = narrow<R>(x);
     }
 #pragma unroll
   for (int m = 0; m < ST::NSUB; m++)
@@ -729,7 +732,7 @@ __device__ __forceinline__ void setup_thread(const ST& st, const double* p, cons
     E e[4];
 #pragma unroll
     for (int mu = 0; mu < 4; mu++) e[mu] = E(k[l][mu]);
-    leg_states<P, R, E>(st, e, kp, l);
+    leg_states<P, R, E>(st, e, kr, l);
   }
 }
 

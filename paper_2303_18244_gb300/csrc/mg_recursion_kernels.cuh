@@ -94,6 +94,7 @@ __device__ __forceinline__ void rec_events(unsigned char* smem, const double* __
   const int tid = threadIdx.x, gt = tid % T, ge = tid / T;
   const int per = blockDim.x / T;
   const ST st(smem + LY::store_off + ge * LY::store_bytes);
+  const R kr[2] = {R(kp.v[0]), R(kp.v[1])};
   const long long step = (long long)gridDim.x * per;
   auto fetch = [&](long long e0) {
     const uint32_t bytes = (uint32_t)((nevt - e0 < per ? nevt - e0 : per) * LY::mom_bytes);
@@ -121,18 +122,23 @@ __device__ __forceinline__ void rec_events(unsigned char* smem, const double* __
     const bool valid = e0 + ge < nevt;
     const long long e = valid ? e0 + ge : nevt - 1;
     const double* pm = reinterpret_cast<const double*>(smem + LY::mom_off) + (e - e0) * P::NPAR * 4;
-    for (int m = gt; m < ST::NSUB; m += T) rec::setup_momenta<P, R, D>(st, pm, m);
-    for (int l = gt; l < P::N + 2; l += T) rec::setup_leg<P, R, D>(st, pm, kp.v, l);
-    if constexpr (sizeof(R) == 4 && sizeof(D) == 8) {
+    constexpr bool pairs = sizeof(R) == 4 && sizeof(D) == 8;
+    R* k = st.momenta();
+    for (int t = gt; t < P::NPAR * 4; t += T) k[t] = rec::narrow<R>(pm[t]);
+    if constexpr (pairs)
       for (int t = gt; t < (P::N + 1) * (P::N + 2) / 2; t += T) rec::setup_pair<P>(st.pairs(), pm, t);
-      __syncthreads();
-      for (int c = gt; c < 2 * ST::NSUB; c += T) rec::setup_coef_pairs<P>(st, st.pairs(), kp.v, c);
-    } else {
-      for (int c = gt; c < 2 * ST::NSUB; c += T) rec::setup_coef<P, R, D>(st, pm, kp.v, c);
+    __syncthreads();
+    for (int m = gt; m < ST::NSUB; m += T) rec::setup_momenta<P, R>(st, k, m);
+    for (int l = gt; l < P::N + 2; l += T) rec::setup_leg<P, R>(st, k, kr, l);
+    for (int c = gt; c < 2 * ST::NSUB; c += T) {
+      if constexpr (pairs)
+        rec::setup_coef_pairs<P>(st, st.pairs(), kp.v, c);
+      else
+        rec::setup_coef<P, R, D>(st, pm, kp.v, c);
     }
     __syncthreads();
     if (tid == 0 && e0 + step < nevt) fetch(e0 + step);  // the momenta are consumed
-    P::template currents<R>(st, kp.v, gt, T, [] { __syncthreads(); });
+    P::template currents<R>(st, kr, gt, T, [] { __syncthreads(); });
     __syncthreads();
     body(st, e, valid);
     __syncthreads();  // the store is rewritten by the next tile
@@ -224,6 +230,8 @@ __global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_
         A v;
         if constexpr (MODE == REC_PAPER)
           v = (A)P::colour_form_paper(f[ib]);
+        else if constexpr (sizeof(R) == 4 && sizeof(A) == 8)
+          v = rec::widen_f64(P::template colour_form<R>(f[ib]));
         else
           v = (A)P::template colour_form<R>(f[ib]);
         const bool in = (good >> (b0 + ib) & 1) != 0;
@@ -275,7 +283,8 @@ __device__ __forceinline__ void rec_cta_flows(const ST& st, const KParams& kp, c
   const int hg = gt & ((1 << P::N) - 1), s = gt >> P::N & 1, b = gt >> (P::N + 1);
   P::template closings<R, 1>(st, hg, s, b, [&](int, int k, cx<R> v) { put(k, v); });
   __syncthreads();
-  P::template late<R>(st, kp.v, gt, P::NHEL);
+  const R kr[2] = {R(kp.v[0]), R(kp.v[1])};
+  P::template late<R>(st, kr, gt, P::NHEL);
   __syncthreads();
   P::template all_flows<R, 1>(
       st, hg, s, b, [&](int, int k) { return get(k); }, [&](int, int k, cx<R> v) { put(k, v); });
@@ -368,10 +377,13 @@ __global__ void __launch_bounds__(RecShape<P, float>::T* RecShape<P, float>::EV,
 }
 
 // Phase 2: one CTA per event at a time, TMEM lane = helicity: FP16 hi/lo
-// operand tiles of the rows, D = A K for Re and Im, sum_k J_k D_k per row with
-// the FP32 flows, and the rows of the list summed in FP64.
+// operand tiles of the rows, D = A K for Re, then Im, sum_k J_k D_k per row with
+// the FP32 flows, and the rows of the list summed in FP64.  The loads of an
+// event (123 KB from HBM) bound it: one part at a time keeps two CTAs on an SM
+// (97 KB of shared memory and half of the tensor memory each), so that one
+// loads while the other converts and contracts.
 template <class P>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(128, 2)
     rec_colour_tc_kernel(const float2* __restrict__ J, long long nevt, double* __restrict__ me,
                          const int* __restrict__ hels, int nhel, const uint4* __restrict__ ctile,
                          unsigned* __restrict__ status, uint32_t polls) {
@@ -415,18 +427,28 @@ __global__ void __launch_bounds__(128, 1)
       fr[k] = v.x;
       fi[k] = v.y;
     }
-    const float s = colour_operands<P, K>(atile, LY::a_tile, tid, fr, fi);
-    fence_proxy_async_smem();  // generic-proxy tile writes -> visible to the tensor core
-    __syncthreads();
-    if (tid == 0) colour_mma<K, N>(tmem, a_addr, b_addr, LY::a_tile, mma_bar);
-    if (!__syncthreads_and(mbar_wait_bounded(mma_bar, phase, polls) ? 1 : 0)) {
-      if (tid == 0) atomicOr(status, ST_MMA_TIMEOUT);
-      ok = false;
-      break;
+    const float s = colour_scale<P, K>(fr, fi);
+    float dsum = 0.f;
+#pragma unroll
+    for (int part = 0; part < 2; part++) {  // Re, then Im
+      colour_operands<P, K>(atile, LY::a_tile, tid, s, part ? fi : fr);
+      fence_proxy_async_smem();  // generic-proxy tile writes -> visible to the tensor core
+      tc::fence_before_sync();
+      __syncthreads();
+      if (tid == 0) colour_mma<K, N>(tmem + part * N, a_addr, b_addr, LY::a_tile, mma_bar);
+      if (part) dsum = colour_readback<P, N>(lane_base, fr);  // Re, while the tensor core works on Im
+      // the outcome of the bounded wait is made uniform across the CTA, so that
+      // no thread can skip the warp-collective TMEM loads or a barrier alone
+      if (!__syncthreads_and(mbar_wait_bounded(mma_bar, phase, polls) ? 1 : 0)) {
+        if (tid == 0) atomicOr(status, ST_MMA_TIMEOUT);
+        ok = false;
+        break;
+      }
+      phase ^= 1u;
+      tc::fence_after_sync();
     }
-    phase ^= 1u;
-    tc::fence_after_sync();
-    const float dsum = colour_readback<P, N>(lane_base, fr, fi);
+    if (!ok) break;
+    dsum += colour_readback<P, N>(lane_base + N, fi);
     const double part = rec_group_sum<32>(good ? (double)(dsum / s) : 0.0, static_cast<double*>(nullptr));
     if ((tid & 31) == 0) red[warp] = part;
     tc::fence_before_sync();
@@ -448,6 +470,13 @@ __global__ void __launch_bounds__(128, 1)
 // ---------------------------------------------------------------------------
 // host-side launchers
 // ---------------------------------------------------------------------------
+inline int rec_sms() {
+  int dev = 0, sms = 0;
+  return cudaGetDevice(&dev) == cudaSuccess &&
+                 cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess
+             ? sms
+             : 0;
+}
 // Resident CTAs of a kernel on the current device: the persistent grid.
 template <class K>
 inline int rec_resident(K kernel, int threads, size_t smem) {
@@ -504,7 +533,9 @@ int launch_rec_rows(const LaunchArgs& a) {
   static const cudaError_t attr2 = set_smem_attr(rec_colour_tc_kernel<P>, smem2);
   if (attr1 != cudaSuccess || attr2 != cudaSuccess) return -4;
   static const int res1 = rec_resident(rec_flows_kernel<P>, LY::T * LY::EV, smem1);
-  static const int res2 = rec_resident(rec_colour_tc_kernel<P>, 128, smem2);
+  // two CTAs per SM (launch bounds, shared and tensor memory; the occupancy
+  // query counts one for a kernel that allocates tensor memory)
+  static const int res2 = 2 * rec_sms();
   if (res1 < 1 || res2 < 1) return -4;
   if (a.nevt <= 0 || a.nhel <= 0) return 0;
 #ifdef MG_REC_SLICE

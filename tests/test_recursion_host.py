@@ -50,9 +50,9 @@ int main() {
       if (scanf("%lf", &x) != 1) return 1;
     std::vector<double> slab(TAG::NSLOT);
     TAG::prepare<double, double>(p, kp, slab.data(), 1);
-    for (int m = 0; m < ST::NSUB; m++) rec::setup_momenta<P, double, double>(st, p, m);
+    for (int m = 0; m < ST::NSUB; m++) rec::setup_momenta<P, double>(st, p, m);
     for (int c = 0; c < 2 * ST::NSUB; c++) rec::setup_coef<P, double, double>(st, p, kp, c);
-    for (int l = 0; l < P::N + 2; l++) rec::setup_leg<P, double, double>(st, p, kp, l);
+    for (int l = 0; l < P::N + 2; l++) rec::setup_leg<P, double>(st, p, kp, l);
     CURRENTS
     for (int hg = 0; hg < (1 << P::N); hg++)
       for (int s = 0; s < 2; s++) {
