@@ -196,11 +196,16 @@ struct Store {
   static constexpr size_t pair_off = vec_bytes + size_t(NS) * sizeof(R);  // setup_pair (FP32)
   static constexpr size_t mom_off = pair_off + (sizeof(R) == 4 ? size_t((N + 1) * (N + 2) / 2) * sizeof(double) : 0);
   static constexpr size_t bytes = mom_off + size_t(N + 2) * 4 * sizeof(R);  // the event's momenta in R
+  static constexpr size_t stride = (bytes + 127) / 128 * 128;               // to the next event's store
   Pack<R>* p;
   R* sc;
   __device__ __forceinline__ explicit Store(void* mem)
       : p(reinterpret_cast<Pack<R>*>(mem)),
         sc(reinterpret_cast<R*>(reinterpret_cast<unsigned char*>(mem) + vec_bytes)) {}
+  // the store e events on
+  __device__ __forceinline__ Store at(int e) const {
+    return Store(reinterpret_cast<unsigned char*>(p) + (ptrdiff_t)e * (ptrdiff_t)stride);
+  }
   __device__ __forceinline__ double* pairs() const {
     return reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(p) + pair_off);
   }
@@ -392,12 +397,10 @@ __device__ __forceinline__ double quick_inverse(double d) {
   const double w = widen_f64(y);
   return fmad(fmad(-d, w, 1.0), w, w);
 }
+// subset m: both of its denominators
 template <class P, class ST>
-__device__ __forceinline__ void setup_coef_pairs(const ST& st, const double* pairs, const double* kp, int c) {
+__device__ __forceinline__ void setup_coef_pairs(const ST& st, const double* pairs, const double* kp, int m) {
   constexpr int N = P::N;
-  if (!is_propagator<N>(c)) return;
-  const bool f = (c >> N) != 0;
-  const int m = c & (ST::NSUB - 1);
   const double g = kp[0], mt = kp[1], wt = kp[2];
   double self = 0.0, mix = 0.0, pk = 0.0;
 #pragma unroll
@@ -410,15 +413,13 @@ __device__ __forceinline__ void setup_coef_pairs(const ST& st, const double* pai
     for (int i = 0; i < j; i++)
       if ((m >> i & 1) && (m >> j & 1)) mix += pairs[pair_at<N>(i + 1, j + 1)];
   }
-  double v;
-  if (f) {
-    v = fmad(2.0, mix - pk, self + (pairs[0] - mt * mt));
-  } else {
-    v = fmad(2.0, mix, self);
+  if (is_propagator<N>(m)) store_coef<float>(st, m, false, round_f32(-g * quick_inverse(fmad(2.0, mix, self))), 0.f);
+  if (is_propagator<N>(m | 1 << N)) {
+    const double v = fmad(2.0, mix - pk, self + (pairs[0] - mt * mt));
+    const double dim = mt * wt;
+    const double r = -g * quick_inverse(fmad(v, v, dim * dim));
+    store_coef<float>(st, m, true, round_f32(r * v), round_f32(-r * dim));
   }
-  const double dim = mt * wt;
-  const double r = -g * quick_inverse(f ? fmad(v, v, dim * dim) : v);
-  store_coef<float>(st, m, f, round_f32(f ? r * v : r), f ? round_f32(-r * dim) : 0.f);
 }
 
 // external states of leg l (gluons, then t, t~) of momentum q
@@ -479,8 +480,16 @@ struct alignas(16) Row {
 //   Q(X, Y, Z) = -g [2 (X.Z) Y - (Y.Z) X - (X.Y) Z].
 // The coefficient of each sub-current is collected first, so that every one
 // is scaled and added once.  Table: the sub-currents [i, j) in (i, j) order,
-// the two masks of every split, the mask of w, the destination (and for
-// pairs the destination of J(w reversed) = -J(w)).
+// the two masks of every split, the destination and that of the current with
+// every helicity flipped, (-1)^m J* (and for pairs the two destinations of
+// J(w reversed) = -J(w)).
+template <typename R>
+__device__ __forceinline__ V4<R> flipped(const V4<R>& a, bool odd) {
+  V4<R> o;
+#pragma unroll
+  for (int mu = 0; mu < 4; mu++) o.c[mu] = {odd ? -a.c[mu].re : a.c[mu].re, odd ? a.c[mu].im : -a.c[mu].im};
+  return o;
+}
 template <int M, typename R, class ST, class RW>
 __device__ __forceinline__ void j_task(const ST& st, const RW& row, const R* kr) {
   constexpr int NSUBW = M * (M + 1) / 2 - 1;
@@ -541,19 +550,23 @@ __device__ __forceinline__ void j_task(const ST& st, const RW& row, const R* kr)
   for (int q = 0; q < NSUBW; q++)
 #pragma unroll
     for (int mu = 0; mu < 4; mu++) cmac(acc.c[mu], c[q], J[q].c[mu]);
-  const R cg = st.sc[ST::S_CG + row.v[NSUBW + 2 * (M - 1)]];
+  constexpr int DST = NSUBW + 2 * (M - 1);
+  const R cg = st.sc[ST::S_CG + (row.v[NSUBW] | row.v[NSUBW + 1])];  // mask of w: of its first split
 #pragma unroll
   for (int mu = 0; mu < 4; mu++) acc.c[mu] = {cg * acc.c[mu].re, cg * acc.c[mu].im};
-  st.st(row.v[NSUBW + 2 * (M - 1) + 1], acc);
+  st.st(row.v[DST], acc);
+  st.st(row.v[DST + 1], flipped(acc, M % 2 != 0));
   if constexpr (M == 2) {
 #pragma unroll
     for (int mu = 0; mu < 4; mu++) acc.c[mu] = -acc.c[mu];
-    st.st(row.v[NSUBW + 2 * (M - 1) + 2], acc);
+    st.st(row.v[DST + 2], acc);
+    st.st(row.v[DST + 3], flipped(acc, false));
   }
 }
 
 // +- the sum of one to three vectors (Kleiss-Kuijf): x1, x2, x3, destination,
-// number of terms, sign flag
+// number of terms, sign flag, destination with every helicity flipped, odd
+// number of gluons
 template <typename R, class ST, class RW>
 __device__ __forceinline__ void comb_task(const ST& st, const RW& row) {
   V4<R> o = st.ld(row.v[0]);
@@ -566,6 +579,7 @@ __device__ __forceinline__ void comb_task(const ST& st, const RW& row) {
   const R sg = row.v[5] ? R(-1) : R(1);
   for (int mu = 0; mu < 4; mu++) o.c[mu] = {sg * o.c[mu].re, sg * o.c[mu].im};
   st.st(row.v[3], o);
+  st.st(row.v[6], flipped(o, row.v[7] != 0));
 }
 
 // amputated line: sum over NT pairs (spinor, current); table: the pairs, destination

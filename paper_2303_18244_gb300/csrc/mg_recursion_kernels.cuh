@@ -25,7 +25,11 @@ struct RecShape {
   // warps of a CTA, a multiple of the four schedulers.  Measured, 524288 events
   // of four gluons in FP32: 5 / 8 / 10 / 12 warps 9.6 / 6.9 / 7.2 / 6.6 ms (12
   // fill the shared memory); three gluons 8 / 12 warps 0.19 / 0.23 ms per 65536;
-  // FP64, 32749 events of four gluons: 4 / 5 warps 12.5 / 13.6 ms.
+  // FP64, 32749 events of four gluons: 4 / 5 warps 12.5 / 13.6 ms.  Since half of
+  // the currents come by conjugation and the lists run over the CTA's events,
+  // several smaller CTAs per SM (which could overlap one's FP64 set-up with
+  // another's closings) still give nothing: 1 x 12 / 2 x 6 / 3 x 4 warps 4.89 /
+  // 4.97 / 5.03 ms; FP64 1 x 4 / 2 x 2 11.22 / 11.20 ms.
   static constexpr int WARPS = P::N == 4 ? (f32 ? 12 : 4) : (f32 ? 8 : 4);
   static constexpr int EV = WARPS * 32 / T;
 };
@@ -39,7 +43,7 @@ struct RecLayout {
   static constexpr size_t red_off = 16;                                       // after the mbarrier: partial sums
   static constexpr size_t mom_off = 128;
   static constexpr size_t store_off = mom_off + r128(EV * mom_bytes);
-  static constexpr size_t store_bytes = r128(ST::bytes);
+  static constexpr size_t store_bytes = ST::stride;
   static constexpr size_t base_bytes = store_off + EV * store_bytes;
 };
 
@@ -82,6 +86,9 @@ __device__ __forceinline__ double warp_scatter_sum(const double (&v)[N]) {
   return x[0];
 }
 
+template <int N>
+using Count = std::integral_constant<int, N>;
+
 // The event loop; blockDim.x = T * (events per tile).  body(store, e, valid)
 // runs with the currents complete; groups past the last event repeat it.
 template <class P, typename R, typename D, class BODY>
@@ -91,9 +98,9 @@ __device__ __forceinline__ void rec_events(unsigned char* smem, const double* __
   using ST = typename LY::ST;
   constexpr int T = LY::T;
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
-  const int tid = threadIdx.x, gt = tid % T, ge = tid / T;
-  const int per = blockDim.x / T;
-  const ST st(smem + LY::store_off + ge * LY::store_bytes);
+  const int tid = threadIdx.x, nt = blockDim.x, ge = tid / T;
+  const int per = nt / T;
+  const ST all(smem + LY::store_off), st = all.at(ge);
   const R kr[2] = {R(kp.v[0]), R(kp.v[1])};
   const long long step = (long long)gridDim.x * per;
   auto fetch = [&](long long e0) {
@@ -121,24 +128,30 @@ __device__ __forceinline__ void rec_events(unsigned char* smem, const double* __
     phase ^= 1u;
     const bool valid = e0 + ge < nevt;
     const long long e = valid ? e0 + ge : nevt - 1;
-    const double* pm = reinterpret_cast<const double*>(smem + LY::mom_off) + (e - e0) * P::NPAR * 4;
+    const double* tile = reinterpret_cast<const double*>(smem + LY::mom_off);
+    const int last = (int)(nevt - e0 < per ? nevt - e0 : per) - 1;
+    auto momenta = [&](int ev) { return tile + (ev < last ? ev : last) * P::NPAR * 4; };
+    // the set-up's tasks of all events of the tile, like the lists of currents
+    auto each = [&](auto count, const auto& task) {
+      constexpr int n = decltype(count)::value;
+      for (int t = tid; t < n * per; t += nt) task(t / n, t % n);
+    };
     constexpr bool pairs = sizeof(R) == 4 && sizeof(D) == 8;
-    R* k = st.momenta();
-    for (int t = gt; t < P::NPAR * 4; t += T) k[t] = rec::narrow<R>(pm[t]);
+    each(Count<P::NPAR * 4>{}, [&](int ev, int t) { all.at(ev).momenta()[t] = rec::narrow<R>(momenta(ev)[t]); });
     if constexpr (pairs)
-      for (int t = gt; t < (P::N + 1) * (P::N + 2) / 2; t += T) rec::setup_pair<P>(st.pairs(), pm, t);
+      each(Count<(P::N + 1) * (P::N + 2) / 2>{},
+           [&](int ev, int t) { rec::setup_pair<P>(all.at(ev).pairs(), momenta(ev), t); });
     __syncthreads();
-    for (int m = gt; m < ST::NSUB; m += T) rec::setup_momenta<P, R>(st, k, m);
-    for (int l = gt; l < P::N + 2; l += T) rec::setup_leg<P, R>(st, k, kr, l);
-    for (int c = gt; c < 2 * ST::NSUB; c += T) {
-      if constexpr (pairs)
-        rec::setup_coef_pairs<P>(st, st.pairs(), kp.v, c);
-      else
-        rec::setup_coef<P, R, D>(st, pm, kp.v, c);
-    }
+    each(Count<ST::NSUB>{}, [&](int ev, int m) { rec::setup_momenta<P, R>(all.at(ev), all.at(ev).momenta(), m); });
+    each(Count<P::N + 2>{}, [&](int ev, int l) { rec::setup_leg<P, R>(all.at(ev), all.at(ev).momenta(), kr, l); });
+    if constexpr (pairs)
+      each(Count<ST::NSUB>{}, [&](int ev, int m) { rec::setup_coef_pairs<P>(all.at(ev), all.at(ev).pairs(), kp.v, m); });
+    else
+      each(Count<2 * ST::NSUB>{},
+           [&](int ev, int c) { rec::setup_coef<P, R, D>(all.at(ev), momenta(ev), kp.v, c); });
     __syncthreads();
     if (tid == 0 && e0 + step < nevt) fetch(e0 + step);  // the momenta are consumed
-    P::template currents<R>(st, kr, gt, T, [] { __syncthreads(); });
+    P::template currents<R>(all, kr, tid, nt, [] { __syncthreads(); }, per);
     __syncthreads();
     body(st, e, valid);
     __syncthreads();  // the store is rewritten by the next tile
@@ -212,7 +225,7 @@ __global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_
     A acc = A(0);
     [[maybe_unused]] double w = 0.0;
     if constexpr (P::LATE && NB == 1) {  // the late vectors have space of their own
-      P::template late<R>(st, gt, T);
+      P::template late<R>(st.at(-ge), threadIdx.x, blockDim.x, blockDim.x / T);
       __syncthreads();
     }
 #pragma unroll 1
@@ -221,7 +234,7 @@ __global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_
       P::template flows_open<R, NB>(st, hg, s, b0, f);
       if constexpr (P::LATE && NB == 2) {  // ... or take that of the vectors just closed
         __syncthreads();
-        P::template late<R>(st, gt, T);
+        P::template late<R>(st.at(-ge), threadIdx.x, blockDim.x, blockDim.x / T);
         __syncthreads();
       }
       P::template flows_block<R, NB>(st, hg, s, b0, f);
@@ -284,7 +297,7 @@ __device__ __forceinline__ void rec_cta_flows(const ST& st, const KParams& kp, c
   P::template closings<R, 1>(st, hg, s, b, [&](int, int k, cx<R> v) { put(k, v); });
   __syncthreads();
   const R kr[2] = {R(kp.v[0]), R(kp.v[1])};
-  P::template late<R>(st, kr, gt, P::NHEL);
+  P::template late<R>(st.at(-(int)(threadIdx.x / P::NHEL)), kr, threadIdx.x, blockDim.x, blockDim.x / P::NHEL);
   __syncthreads();
   P::template all_flows<R, 1>(
       st, hg, s, b, [&](int, int k) { return get(k); }, [&](int, int k, cx<R> v) { put(k, v); });

@@ -82,7 +82,7 @@ using ST = rec::Store<Cnt, P::N, P::NVEC<Cnt>>;
 int main() {
   std::vector<Cnt> mem(ST::bytes / sizeof(Cnt) + 16, Cnt(0.01));
   const ST st(reinterpret_cast<void*>((reinterpret_cast<size_t>(mem.data()) + 15) / 16 * 16));
-  double kp[8] = {1.2, 173.0, 1.5, 0, 0, 0, 0, 0};
+  const Cnt kp[8] = {1.2, 173.0, 1.5, 0, 0, 0, 0, 0};
   long long colour = 0;
   CURRENTS
   for (int hg = 0; hg < (1 << P::N); hg++)

@@ -14,7 +14,12 @@ store:
              words that start with their smallest gluon; the other orders
              follow from the Kleiss-Kuijf relation
              J(a, m, b) = (-1)^|a| sum over shuffles s of (a reversed, b) J(m, s)
-             (R. Kleiss, H. Kuijf, Nucl. Phys. B312 (1989) 616)
+             (R. Kleiss, H. Kuijf, Nucl. Phys. B312 (1989) 616).  Momenta,
+             couplings and gluon propagators are real and
+             eps(-lambda) = -eps(lambda)*, so the current of m gluons with every
+             helicity flipped is (-1)^m J*, bit for bit: half of the helicity
+             combinations are computed, each writes its partner too (the lines
+             have no such partners: the top's width is complex)
   R(word)    row spinor that left the outgoing top and absorbed `word`
   A(word)    the same before the last propagator (amputated)
   C(word)    column spinor that ends on the antitop, stored as the row of its
@@ -255,12 +260,20 @@ class Recursion:
             else:
                 yield hel, spin, spin
 
+    def _task_combos(self, key):
+        """Combinations that have a task of their own: of the gluon currents
+        the half whose last gluon has helicity bit 0."""
+        for hel, s, b in self._combos(key):
+            if key[0] != "J" or not hel[self.items[key][0][-1]]:
+                yield hel, s, b
+
     # -- task tables -------------------------------------------------------
     def table(self, stage, keys):
         """Rows of 16-bit numbers, one per task (item x helicity combination)."""
         rows = []
         for key in keys:
-            for hel, s, b in self._combos(key):
+            for hel, s, b in self._task_combos(key):
+                flip = {g: 1 - x for g, x in hel.items()}
                 ix = lambda k: self.index(k, hel, s, b)  # noqa: E731
                 dst = ix(key)
                 if stage[0] == "J":
@@ -269,13 +282,14 @@ class Recursion:
                     row = [ix(self.jkey(w[i:j])) for i in range(m) for j in range(i + 1, m + 1) if j - i < m]
                     for i in range(1, m):
                         row += [self.mask(w[:i]), self.mask(w[i:])]
-                    row += [self.mask(w), dst]
+                    row += [dst, self.index(key, flip)]
                     if m == 2:
-                        row.append(ix(self.jkey(w[::-1])))
+                        row += [self.index(self.jkey(w[::-1]), x) for x in (hel, flip)]
                 elif stage[0] == "K":
                     sg, ws = kk(key[1])
                     row = [ix(self.jkey(w)) for w in ws]
                     row += [row[0]] * (3 - len(row)) + [dst, len(ws), 1 if sg < 0 else 0]
+                    row += [self.index(key, flip), len(key[1]) % 2]
                 elif stage[0] in "RAC":
                     w = key[1]
                     m = len(w)
@@ -319,8 +333,15 @@ class Recursion:
         return [k for i in range(m) for k in (("R", w[:i]), self.jkey(w[i:]))]
 
     def level(self, key) -> int:
+        """Stage of an item.  The currents of one length are one list (their
+        code is the longest, so it is there and fetched once), the Kleiss-Kuijf
+        sums of one length another."""
         if key not in self._lev:
-            self._lev[key] = 1 + max([self.level(k) for k in self.deps(key)], default=-1)
+            w = key[1]
+            group = [key]
+            if key[0] == "J" and len(w) > 2:
+                group = self.tasks[("J" if w[0] == min(w) else "K") + str(len(w))]
+            self._lev[key] = 1 + max([self.level(d) for k in group for d in self.deps(k)], default=-1)
         return self._lev[key]
 
     def routine(self, key) -> str:
@@ -582,7 +603,7 @@ def _thread_sum(rec: Recursion) -> list[str]:
     for stage, keys in rec.tasks.items():
         for key in keys:
             rows = rec.table(stage, [key])
-            for row, (hel, s, b) in zip(rows, rec._combos(key)):
+            for row, (hel, s, b) in zip(rows, rec._task_combos(key), strict=True):
                 w = ((len(row) + 7) // 8) * 8
                 lit = f"Row<{w}>{{{{" + ", ".join(str(x) for x in row + [0] * (w - len(row))) + "}}"
                 when = b if key[0] in "CV" else None
@@ -615,7 +636,8 @@ def _grouped_flows(rec: Recursion, head, tag, late) -> list[str]:
     L = []
     L.append("  // columns of three gluons, over the store space that closings() read")
     L.append("  template <typename R, class ST>")
-    L.append("  __device__ static __forceinline__ void late(const ST& st, const R* kr, const int tid, const int nt) {")
+    L.append("  __device__ static __forceinline__ void late(const ST& all, const R* kr, const int tid, const int nt,")
+    L.append("                                              const int per = 1) {")
     L += late
     L.append("  }")
     em = _Emit(rec)
@@ -745,7 +767,9 @@ def emit_recursion(n: int, tag: str) -> str:
     # five gluons: a task's table line is fetched one task ahead, a list's first
     # one before the barrier of its stage (60 KB of lines come from L2: the store
     # leaves little L1; 8229 mixed events, flow kernel 1.49 -> 1.44 ms; the
-    # smaller tables stay in L1, where it cost FP64 2 %)
+    # smaller tables stay in L1, where it cost FP64 2 %).  A list runs over the
+    # tasks of all events of the CTA, so that its last, partly filled round is
+    # one of the CTA and not one of every warp.
     levels: dict = {}
     for q, (lev, fn, rows) in enumerate(rec.stages()):
         w = ((len(rows[0]) + 7) // 8) * 8
@@ -756,14 +780,16 @@ def emit_recursion(n: int, tag: str) -> str:
                  + ", ".join("{{" + ", ".join(str(x) for x in flat[i:i + w]) + "}}" for i in range(0, len(flat), w))
                  + "};")
         if n < 5:
-            levels.setdefault(lev, []).append((None, [f"    MG_REC_LOOP for (int t = tid; t < {len(rows)}; t += nt) "
-                                                      f"{fn.format(row=f'{name}[t]')};"]))
+            levels.setdefault(lev, []).append((None, [
+                f"    MG_REC_LOOP for (int t = tid; t < {len(rows)} * per; t += nt) {{",
+                f"      const ST st = all.at(t / {len(rows)});",
+                f"      {fn.format(row=f'{name}[t % {len(rows)}]')};", "    }"]))
             continue
         levels.setdefault(lev, []).append((
-            f"    rec::Row<{w}> r{q} = {name}[tid < {len(rows)} ? tid : {len(rows) - 1}];",
-            [f"    MG_REC_LOOP for (int t = tid; t < {len(rows)}; t += nt) {{",
-             f"      const rec::Row<{w}> row = r{q};",
-             f"      if (t + nt < {len(rows)}) r{q} = {name}[t + nt];",
+            f"    rec::Row<{w}> r{q} = {name}[tid % {len(rows)}];",
+            [f"    MG_REC_LOOP for (int t = tid; t < {len(rows)} * per; t += nt) {{",
+             f"      const rec::Row<{w}> row = r{q};", f"      const ST st = all.at(t / {len(rows)});",
+             f"      r{q} = {name}[(t + nt) % {len(rows)}];",
              f"      {fn.format(row='row')};", "    }"]))
     for lev in sorted(levels):
         out = late if lev == 99 else body
@@ -795,9 +821,10 @@ def emit_recursion(n: int, tag: str) -> str:
     L.append(f"    for (int i = 0; i < {n}; i++) h |= (hg >> i & 1) << ({n + 1} - (i < 2 ? i : i + 2));")
     L.append("    return h;")
     L.append("  }")
+    L.append("  // the currents of `per` events (all: the store of the first), by nt threads")
     L.append("  template <typename R, class ST, class SYNC>")
-    L.append("  __device__ static __forceinline__ void currents(const ST& st, const R* kr, const int tid, const int nt,")
-    L.append("                                                  const SYNC& sync) {")
+    L.append("  __device__ static __forceinline__ void currents(const ST& all, const R* kr, const int tid, const int nt,")
+    L.append("                                                  const SYNC& sync, const int per = 1) {")
     L += body
     L.append("  }")
     if n <= 4:
@@ -807,8 +834,9 @@ def emit_recursion(n: int, tag: str) -> str:
             L.append(f"  static constexpr int S0 = sizeof(R) == 4 ? 0 : {rec.nvec};")
         L.append(f"  static constexpr bool LATE = {'true' if late else 'false'};")
         L.append("  template <typename R, class ST>")
-        L.append("  __device__ static __forceinline__ void late([[maybe_unused]] const ST& st, [[maybe_unused]] const int tid,")
-        L.append("                                              [[maybe_unused]] const int nt) {")
+        L.append("  __device__ static __forceinline__ void late([[maybe_unused]] const ST& all, [[maybe_unused]] const int tid,")
+        L.append("                                              [[maybe_unused]] const int nt,")
+        L.append("                                              [[maybe_unused]] const int per = 1) {")
         L += late
         L.append("  }")
         flows = {w: i for i, w in enumerate(ws)}
