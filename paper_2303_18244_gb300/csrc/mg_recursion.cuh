@@ -359,20 +359,21 @@ __device__ __forceinline__ void setup_coef(const ST& st, const double* p, const 
 // The same for FP32 amplitudes with FP64 denominators, with a third of the
 // FP64 instructions (GB300's FP64 pipe takes 16 cycles per warp instruction;
 // the plain form kept it busy for a third of the four-gluon kernel): first
-// the products of every pair of the momenta p_t, k_0 .. k_N-1 (incoming), then
-//   K^2 = sum k_i^2 + 2 sum k_i.k_j,
-//   (p_t - K)^2 - m^2 = p_t^2 - m^2 + K^2 - 2 sum p_t.k_i,
+// the products p_t^2 - m^2, k_i^2 and twice those of every other pair of the
+// momenta p_t, k_0 .. k_N-1 (incoming), then
+//   K^2 = sum k_i^2 + sum 2 k_i.k_j,
+//   (p_t - K)^2 - m^2 = (p_t^2 - m^2 - sum 2 p_t.k_i) + K^2,
 // which rounds like the square of the sum (a few 1e-16 of the largest energy
 // squared; masses and on-shell conditions are not assumed), and 1 / d from
 // the FP32 reciprocal and one Newton step (1e-14, then rounded to FP32).
 // pairs: scratch of (N + 1) (N + 2) / 2 doubles; entry j (j + 1) / 2 + i for i <= j,
-// 0: p_t, 1 + i: k_i.
+// 0: p_t, 1 + i: k_i.  kp: g_s, m_t, width, m_t^2, m_t width, (m_t width)^2.
 template <int N>
 __host__ __device__ constexpr int pair_at(int i, int j) {
   return j * (j + 1) / 2 + i;
 }
 template <class P>
-__device__ __forceinline__ void setup_pair(double* pairs, const double* p, int t) {
+__device__ __forceinline__ void setup_pair(double* pairs, const double* p, const double* kp, int t) {
   constexpr int N = P::N;
   if (t >= (N + 1) * (N + 2) / 2) return;
   int j = 0;
@@ -382,13 +383,14 @@ __device__ __forceinline__ void setup_pair(double* pairs, const double* p, int t
   auto in = [](int q) { return q == 0 || q > 2; };                         // outgoing momentum
   const double* a = p + 4 * at(i);
   const double* b = p + 4 * at(j);
-  double d = a[0] * b[0];
+  double d = fmad(a[0], b[0], t == 0 ? -kp[3] : 0.0);
   d = fmad(-a[1], b[1], d);
   d = fmad(-a[2], b[2], d);
   d = fmad(-a[3], b[3], d);
   // k = -p for the outgoing gluons; p_t as it is
   const bool minus = (i > 0 && in(i)) != (j > 0 && in(j));
-  pairs[t] = minus ? -d : d;
+  d = minus ? -d : d;
+  pairs[t] = i == j ? d : d + d;
 }
 __device__ __forceinline__ double quick_inverse(double d) {
   const float f = round_f32(d);
@@ -401,24 +403,23 @@ __device__ __forceinline__ double quick_inverse(double d) {
 template <class P, class ST>
 __device__ __forceinline__ void setup_coef_pairs(const ST& st, const double* pairs, const double* kp, int m) {
   constexpr int N = P::N;
-  const double g = kp[0], mt = kp[1], wt = kp[2];
-  double self = 0.0, mix = 0.0, pk = 0.0;
+  const double g = kp[0];
+  double v = 0.0, f = pairs[0];
 #pragma unroll
   for (int j = 0; j < N; j++) {
     if (m >> j & 1) {
-      self += pairs[pair_at<N>(j + 1, j + 1)];
-      pk += pairs[pair_at<N>(0, j + 1)];
+      v += pairs[pair_at<N>(j + 1, j + 1)];
+      f -= pairs[pair_at<N>(0, j + 1)];
     }
 #pragma unroll
     for (int i = 0; i < j; i++)
-      if ((m >> i & 1) && (m >> j & 1)) mix += pairs[pair_at<N>(i + 1, j + 1)];
+      if ((m >> i & 1) && (m >> j & 1)) v += pairs[pair_at<N>(i + 1, j + 1)];
   }
-  if (is_propagator<N>(m)) store_coef<float>(st, m, false, round_f32(-g * quick_inverse(fmad(2.0, mix, self))), 0.f);
+  if (is_propagator<N>(m)) store_coef<float>(st, m, false, round_f32(-g * quick_inverse(v)), 0.f);
   if (is_propagator<N>(m | 1 << N)) {
-    const double v = fmad(2.0, mix - pk, self + (pairs[0] - mt * mt));
-    const double dim = mt * wt;
-    const double r = -g * quick_inverse(fmad(v, v, dim * dim));
-    store_coef<float>(st, m, true, round_f32(r * v), round_f32(-r * dim));
+    f += v;
+    const double r = -g * quick_inverse(fmad(f, f, kp[5]));
+    store_coef<float>(st, m, true, round_f32(r * f), round_f32(-r * kp[4]));
   }
 }
 
@@ -722,20 +723,23 @@ __device__ __forceinline__ void setup_thread(const ST& st, const double* p, cons
     st.sc[ST::S_PT + mu] = k[N][mu];
     st.sc[ST::S_PT + 4 + mu] = k[N + 1][mu];
   }
-  const D g = D(kp[0]), mt = D(kp[1]), dim = mt * D(kp[2]);
+  constexpr bool mixed = sizeof(R) == 4 && sizeof(D) == 8;
+  const D g = D(kp[0]), mt = D(kp[1]);
+  const D mt2 = mixed ? D(kp[3]) : mt * mt, dim = mixed ? D(kp[4]) : mt * D(kp[2]);
+  const D dim2 = mixed ? D(kp[5]) : dim * dim;
 #pragma unroll
   for (int c = 0; c < 2 * ST::NSUB; c++) {
     const bool f = (c >> N) != 0;
     const int m = c & (ST::NSUB - 1);
     if (!is_propagator<N>(c)) continue;
-    const D v = subset_mass2<N, R, D>(q, f, m, f ? mt * mt : D(0));
-    const D den = f ? fmad(v, v, dim * dim) : v;
+    const D v = subset_mass2<N, R, D>(q, f, m, f ? mt2 : D(0));
+    const D den = f ? fmad(v, v, dim2) : v;
     D r;
-    if constexpr (sizeof(R) == 4 && sizeof(D) == 8)
+    if constexpr (mixed)
       r = -g * quick_inverse(den);
     else
       r = -g / den;
-    if constexpr (sizeof(R) == 4 && sizeof(D) == 8)
+    if constexpr (mixed)
       store_coef<float>(st, m, f, f ? round_f32(r * v) : round_f32(r), f ? round_f32(-r * dim) : 0.f);
     else
       store_coef<R>(st, m, f, f ? R(r * v) : R(r), R(-r * dim));

@@ -66,6 +66,23 @@ __device__ __forceinline__ A rec_group_sum(A v, A* red) {
   return v;
 }
 
+template <int T>
+__device__ __forceinline__ double rec_group_sum(PairSum v) {
+  static_assert(T <= 32, "within a warp");
+#pragma unroll
+  for (int o = T / 2; o > 0; o >>= 1) {
+    PairSum x;
+    x.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
+    x.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
+    v.add(x);
+  }
+  return v.value();
+}
+template <int T, typename A>
+__device__ __forceinline__ A rec_group_sum(const PlainSum<A>& v) {
+  return rec_group_sum<T>(v.v, static_cast<A*>(nullptr));
+}
+
 // reduce-scatter of N <= 32 values over a warp: lane k < N returns the sum
 // over the lanes of their v[k] (31 additions instead of 5 per value)
 template <int N>
@@ -140,7 +157,7 @@ __device__ __forceinline__ void rec_events(unsigned char* smem, const double* __
     each(Count<P::NPAR * 4>{}, [&](int ev, int t) { all.at(ev).momenta()[t] = rec::narrow<R>(momenta(ev)[t]); });
     if constexpr (pairs)
       each(Count<(P::N + 1) * (P::N + 2) / 2>{},
-           [&](int ev, int t) { rec::setup_pair<P>(all.at(ev).pairs(), momenta(ev), t); });
+           [&](int ev, int t) { rec::setup_pair<P>(all.at(ev).pairs(), momenta(ev), kp.v, t); });
     __syncthreads();
     each(Count<ST::NSUB>{}, [&](int ev, int m) { rec::setup_momenta<P, R>(all.at(ev), all.at(ev).momenta(), m); });
     each(Count<P::N + 2>{}, [&](int ev, int l) { rec::setup_leg<P, R>(all.at(ev), all.at(ev).momenta(), kr, l); });
@@ -222,7 +239,8 @@ __global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_
   double* wk = mh + P::NHEL;
   rec_events<P, R, D>(smem, a.mom, a.nevt, a.kp, a.status, [&](const auto& st, long long e, bool valid) {
     constexpr double norm = 1.0 / (P::IDEN * P::CDEN);
-    A acc = A(0);
+    HelicitySum<R, A> part;
+    [[maybe_unused]] A acc = A(0);
     [[maybe_unused]] double w = 0.0;
     if constexpr (P::LATE && NB == 1) {  // the late vectors have space of their own
       P::template late<R>(st.at(-ge), threadIdx.x, blockDim.x, blockDim.x / T);
@@ -240,18 +258,16 @@ __global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_
       P::template flows_block<R, NB>(st, hg, s, b0, f);
 #pragma unroll
       for (int ib = 0; ib < NB; ib++) {
-        A v;
+        R v;
         if constexpr (MODE == REC_PAPER)
-          v = (A)P::colour_form_paper(f[ib]);
-        else if constexpr (sizeof(R) == 4 && sizeof(A) == 8)
-          v = rec::widen_f64(P::template colour_form<R>(f[ib]));
+          v = (R)P::colour_form_paper(f[ib]);
         else
-          v = (A)P::template colour_form<R>(f[ib]);
+          v = P::template colour_form<R>(f[ib]);
         const bool in = (good >> (b0 + ib) & 1) != 0;
         if constexpr (MODE == REC_HELICITIES) {
           if (valid) a.out[e * P::NHEL + P::helicity(hg, s, b0 + ib)] = (double)v * norm;
         } else if (in) {
-          acc += v;
+          part.add(v);
         }
         if constexpr (MODE == REC_SELECT) {
           static_assert(T <= 32 && P::NCOL <= T, "thread k of the group sums flow k");
@@ -273,7 +289,7 @@ __global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_
       }
     }
     if constexpr (MODE != REC_HELICITIES) {
-      acc = rec_group_sum<T>(acc, static_cast<A*>(nullptr));
+      acc = rec_group_sum<T>(part);
       if (gt == 0 && valid) a.out[e] = (double)(acc * A(norm));
     }
     if constexpr (MODE == REC_SELECT) {

@@ -90,6 +90,10 @@ static int make_kparams(const ProcDesc* d, const mg_params& p, KParams& kp) {
     kp.v[0] = std::sqrt(4.0 * 3.14159265358979323846 * p.alpha_s);  // g_s
     kp.v[1] = p.mt;
     kp.v[2] = (p.flags & MG_NO_TOP_WIDTH) ? 0.0 : p.wt;
+    // of the mixed mode's set-up (every FP64 instruction there counts)
+    kp.v[3] = p.mt * p.mt;
+    kp.v[4] = p.mt * kp.v[2];
+    kp.v[5] = kp.v[4] * kp.v[4];
   }
   return MG_OK;
 }
