@@ -594,8 +594,8 @@ __device__ __forceinline__ V4<R> line_sum(const ST& st, const RW& row) {
   return o;
 }
 template <int NT, typename R, class ST, class RW>
-__device__ __forceinline__ void amp_task(const ST& st, const RW& row, int dst0 = 0) {
-  st.st(dst0 + row.v[2 * NT], line_sum<NT, R>(st, row));
+__device__ __forceinline__ void amp_task(const ST& st, const RW& row) {
+  st.st(row.v[2 * NT], line_sum<NT, R>(st, row));
 }
 // full line; table: the pairs, destination, line (0 top, 1 antitop), mask of
 // the momenta it absorbed, mask of the denominator

@@ -19,18 +19,23 @@ namespace mg {
 template <class P, typename R>
 struct RecShape {
   static constexpr bool f32 = sizeof(R) == 4;
-  // up to four gluons: thread = gluon helicities x top spin, both antitop
-  // spins; five: thread = helicity
-  static constexpr int T = P::N <= 4 ? 1 << (P::N + 1) : P::NHEL;
+  // Thread = gluon helicities x top spin, both antitop spins; or thread =
+  // helicity: five gluons (registers), and four in FP64, where the flows of one
+  // helicity leave room for 12 warps (six events, the late vectors over others)
+  // instead of 4, and 12 keep the FP64 pipe busier: 32749 events 11.3 -> 9.97 ms
+  // (8 / 10 warps 10.2 / 10.5).  In FP32 the antitop spins share the loads of
+  // the rows: 4.66 ms for 524288 events against 5.8 / 5.5 / 5.4 ms with a thread
+  // per helicity and 24 / 20 / 16 warps.  Three gluons, FP64, 65536 events: 2.88
+  // against 2.92 .. 3.6 ms.
+  static constexpr int T = P::N == 5 || (P::N == 4 && !f32) ? P::NHEL : 1 << (P::N + 1);
   // warps of a CTA, a multiple of the four schedulers.  Measured, 524288 events
-  // of four gluons in FP32: 5 / 8 / 10 / 12 warps 9.6 / 6.9 / 7.2 / 6.6 ms (12
-  // fill the shared memory); three gluons 8 / 12 warps 0.19 / 0.23 ms per 65536;
-  // FP64, 32749 events of four gluons: 4 / 5 warps 12.5 / 13.6 ms.  Since half of
-  // the currents come by conjugation and the lists run over the CTA's events,
-  // several smaller CTAs per SM (which could overlap one's FP64 set-up with
-  // another's closings) still give nothing: 1 x 12 / 2 x 6 / 3 x 4 warps 4.89 /
-  // 4.97 / 5.03 ms; FP64 1 x 4 / 2 x 2 11.22 / 11.20 ms.
-  static constexpr int WARPS = P::N == 4 ? (f32 ? 12 : 4) : (f32 ? 8 : 4);
+  // of four gluons in FP32 (with every current computed, before half of them
+  // came by conjugation): 5 / 8 / 10 / 12 warps 9.6 / 6.9 / 7.2 / 6.6 ms; 12
+  // fill the shared memory.  Several smaller CTAs per SM, which could overlap
+  // one's FP64 set-up with another's closings, give nothing: 1 x 12 / 2 x 6 /
+  // 3 x 4 warps 4.89 / 4.97 / 5.03 ms.  Three gluons 8 / 12 warps 0.19 / 0.23 ms
+  // per 65536.
+  static constexpr int WARPS = P::N == 4 ? 12 : f32 ? 8 : 4;
   static constexpr int EV = WARPS * 32 / T;
 };
 
@@ -41,7 +46,7 @@ struct RecLayout {
   static constexpr size_t r128(size_t b) { return (b + 127) / 128 * 128; }
   static constexpr size_t mom_bytes = size_t(P::NPAR) * 4 * sizeof(double);  // per event
   static constexpr size_t red_off = 16;                                       // after the mbarrier: partial sums
-  static constexpr size_t mom_off = 128;
+  static constexpr size_t mom_off = r128(red_off + RecShape<P, R>::WARPS * sizeof(double));
   static constexpr size_t store_off = mom_off + r128(EV * mom_bytes);
   static constexpr size_t store_bytes = ST::stride;
   static constexpr size_t base_bytes = store_off + EV * store_bytes;
@@ -67,20 +72,30 @@ __device__ __forceinline__ A rec_group_sum(A v, A* red) {
 }
 
 template <int T>
-__device__ __forceinline__ double rec_group_sum(PairSum v) {
-  static_assert(T <= 32, "within a warp");
+__device__ __forceinline__ double rec_group_sum(PairSum v, void* red) {
 #pragma unroll
-  for (int o = T / 2; o > 0; o >>= 1) {
+  for (int o = (T < 32 ? T : 32) / 2; o > 0; o >>= 1) {
     PairSum x;
     x.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
     x.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
     v.add(x);
   }
+  if constexpr (T > 32) {
+    constexpr int NW = T / 32;
+    PairSum* slot = static_cast<PairSum*>(red);
+    const int warp = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) slot[warp] = v;
+    __syncthreads();
+    v = PairSum{};
+#pragma unroll
+    for (int w = 0; w < NW; w++) v.add(slot[warp / NW * NW + w]);
+    __syncthreads();
+  }
   return v.value();
 }
 template <int T, typename A>
-__device__ __forceinline__ A rec_group_sum(const PlainSum<A>& v) {
-  return rec_group_sum<T>(v.v, static_cast<A*>(nullptr));
+__device__ __forceinline__ A rec_group_sum(const PlainSum<A>& v, void* red) {
+  return rec_group_sum<T>(v.v, static_cast<A*>(red));
 }
 
 // reduce-scatter of N <= 32 values over a warp: lane k < N returns the sum
@@ -222,35 +237,32 @@ enum RecMode {
   REC_SELECT       // |M|^2 with the helicity and colour choice
 };
 
-// Up to four gluons: the flows of a helicity fit in registers.  FP32 closes
-// both antitop spins at once (they share every load that does not depend on
-// the antitop), FP64 one after the other (registers).
+// Up to four gluons: the flows of a helicity fit in registers.  A thread has a
+// helicity of its own, or both antitop spins: at once in FP32 (they share every
+// load that does not depend on the antitop), one after the other in FP64.
 template <class P, typename R, typename D, typename A, RecMode MODE>
 __global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_kernel(LaunchArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   using LY = RecLayout<P, R>;
-  constexpr int T = LY::T, NB = sizeof(R) == 4 ? 2 : 1;
+  constexpr int T = LY::T, NW = T > 32 ? T / 32 : 1;
+  constexpr bool own = T == P::NHEL;  // a helicity of one's own
+  constexpr int NB = sizeof(R) == 4 && !own ? 2 : 1;
+  static_assert(own || NB == 2 || !P::LATE, "every helicity's first closings come before the late vectors");
   const int gt = threadIdx.x % T, ge = threadIdx.x / T;
-  const int hg = gt & ((1 << P::N) - 1), s = gt >> P::N;
+  const int hg = gt & ((1 << P::N) - 1), s = gt >> P::N & 1;
   unsigned good = 0;
   if constexpr (MODE != REC_HELICITIES) good = rec_good_bits<P>(a.hels, a.nhel, hg, s);
-  // choice: the helicities' values and the flow weights of each event
-  double* mh = reinterpret_cast<double*>(smem + LY::base_bytes) + ge * (P::NHEL + P::NCOL);
+  // choice: the helicities' values and the flow weights (of each warp) of each event
+  double* mh = reinterpret_cast<double*>(smem + LY::base_bytes) + ge * (P::NHEL + NW * P::NCOL);
   double* wk = mh + P::NHEL;
   rec_events<P, R, D>(smem, a.mom, a.nevt, a.kp, a.status, [&](const auto& st, long long e, bool valid) {
     constexpr double norm = 1.0 / (P::IDEN * P::CDEN);
     HelicitySum<R, A> part;
-    [[maybe_unused]] A acc = A(0);
     [[maybe_unused]] double w = 0.0;
-    if constexpr (P::LATE && NB == 1) {  // the late vectors have space of their own
-      P::template late<R>(st.at(-ge), threadIdx.x, blockDim.x, blockDim.x / T);
-      __syncthreads();
-    }
-#pragma unroll 1
-    for (int b0 = 0; b0 < 2; b0 += NB) {
+    const auto close = [&](const int b0) {
       cx<R> f[NB][P::NCOL];
       P::template flows_open<R, NB>(st, hg, s, b0, f);
-      if constexpr (P::LATE && NB == 2) {  // ... or take that of the vectors just closed
+      if constexpr (P::LATE) {  // takes the space of the vectors just closed
         __syncthreads();
         P::template late<R>(st.at(-ge), threadIdx.x, blockDim.x, blockDim.x / T);
         __syncthreads();
@@ -270,13 +282,13 @@ __global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_
           part.add(v);
         }
         if constexpr (MODE == REC_SELECT) {
-          static_assert(T <= 32 && P::NCOL <= T, "thread k of the group sums flow k");
+          static_assert(P::NCOL <= (T < 32 ? T : 32), "lane k of the group sums flow k");
           mh[P::helicity(hg, s, b0 + ib)] = (double)v;
           double sq[P::NCOL];
 #pragma unroll
           for (int k = 0; k < P::NCOL; k++)
             sq[k] = in ? f[ib][k].re * f[ib][k].re + f[ib][k].im * f[ib][k].im : 0.0;
-          if constexpr (T == 32) {
+          if constexpr (T >= 32) {
             w += warp_scatter_sum(sq);
           } else {
 #pragma unroll
@@ -287,19 +299,30 @@ __global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_
           }
         }
       }
+    };
+    if constexpr (own) {
+      close(gt >> (P::N + 1));
+    } else {
+#pragma unroll 1
+      for (int b0 = 0; b0 < 2; b0 += NB) close(b0);
     }
     if constexpr (MODE != REC_HELICITIES) {
-      acc = rec_group_sum<T>(part);
+      const A acc = rec_group_sum<T>(part, smem + LY::red_off);
       if (gt == 0 && valid) a.out[e] = (double)(acc * A(norm));
-    }
-    if constexpr (MODE == REC_SELECT) {
-      if (gt < P::NCOL) {
-        wk[gt] = w;
-        if (a.colw_out && valid) a.colw_out[e * P::NCOL + gt] = w;
+      if constexpr (MODE == REC_SELECT) {
+        const int lane = gt & 31;
+        if (lane < P::NCOL) wk[(gt >> 5) * P::NCOL + lane] = w;
+        __syncthreads();
+        if (gt < P::NCOL) {
+#pragma unroll
+          for (int q = 1; q < NW; q++) w += wk[q * P::NCOL + gt];
+          wk[gt] = w;
+          if (a.colw_out && valid) a.colw_out[e * P::NCOL + gt] = w;
+        }
+        __syncwarp();
+        if (gt == 0 && valid) a.hel_out[e] = rec_choose_helicity(mh, a.hels, a.nhel, a.rnd[2 * e] * (double)acc);
+        if (gt == 1 && valid) a.col_out[e] = rec_choose_flow<P::NCOL>(wk, a.rnd[2 * e + 1]);
       }
-      __syncwarp();
-      if (gt == 0 && valid) a.hel_out[e] = rec_choose_helicity(mh, a.hels, a.nhel, a.rnd[2 * e] * (double)acc);
-      if (gt == 1 && valid) a.col_out[e] = rec_choose_flow<P::NCOL>(wk, a.rnd[2 * e + 1]);
     }
   });
 }
@@ -535,7 +558,9 @@ template <class P, typename R, typename D, typename A, RecMode MODE = REC_SIGMA>
 int launch_rec(const LaunchArgs& a) {
   using LY = RecLayout<P, R>;
   constexpr size_t smem =
-      LY::base_bytes + (MODE == REC_SELECT && P::N <= 4 ? LY::EV * (P::NHEL + P::NCOL) * sizeof(double) : 0);
+      LY::base_bytes + (MODE == REC_SELECT && P::N <= 4
+                            ? LY::EV * (P::NHEL + (LY::T > 32 ? LY::T / 32 : 1) * P::NCOL) * sizeof(double)
+                            : 0);
   constexpr auto kernel = [] {
     if constexpr (P::N <= 4)
       return rec_kernel<P, R, D, A, MODE>;

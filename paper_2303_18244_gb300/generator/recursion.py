@@ -42,13 +42,18 @@ CUT = {2: 1, 3: 1, 4: 2, 5: 2}
 
 # the calls that run an emitted header with one thread (host tests), by
 # n > 4: currents and flows a[2][NCOL] of gluon bits hg and top spin s
-HOST_CURRENTS = ("P::currents<double>(st, kp, 0, 1, [] {});\n    P::late<double>(st, 0, 1);",
+HOST_CURRENTS = ("""P::currents<double>(st, kp, 0, 1, [] {});
+    static cx<double> z[32][2][P::NCOL];
+    for (int q = 0; q < 2 << P::N; q++)
+      P::flows_open<double, 2>(st, q & ((1 << P::N) - 1), q >> P::N, 0, z[q]);
+    P::late<double>(st, 0, 1);""",
                  """P::currents<double>(st, kp, 0, 1, [] {});
     static cx<double> z[64][2][P::NCOL];
     for (int q = 0; q < 64; q++)
       P::closings<double, 2>(st, q & 31, q >> 5, 0, [&](int ib, int k, cx<double> v) { z[q][ib][k] = v; });
     P::late<double>(st, kp, 0, 1);""")
-HOST_FLOWS = ("P::flows_open<double, 2>(st, hg, s, 0, a);\n        P::flows_block<double, 2>(st, hg, s, 0, a);",
+HOST_FLOWS = ("""for (int q = 0; q < 2 * P::NCOL; q++) a[q / P::NCOL][q % P::NCOL] = z[hg + (s << P::N)][q / P::NCOL][q % P::NCOL];
+        P::flows_block<double, 2>(st, hg, s, 0, a);""",
               """const int q = hg + 32 * s;
         P::all_flows<double, 2>(st, hg, s, 0, [&](int ib, int k) { return z[q][ib][k]; },
                                 [&](int ib, int k, cx<double> v) { a[ib][k] = v; });""")
@@ -197,9 +202,7 @@ class Recursion:
     def _layout(self):
         """Store positions.  Items written after others are dead share space
         (`late`).  Four gluons: the spinors S, over A and C of two gluons, once
-        the flows without a block across the cut are closed (FP32; where the
-        registers do not hold the flows meanwhile, S has space of its own at
-        the end).  Five: the columns C of three gluons, over the currents that
+        the flows without a block across the cut are closed.  Five: the columns C of three gluons, over the currents that
         only the full-length closing and the longer currents read."""
         def dead_early(key):
             m = len(key[1])
@@ -354,7 +357,7 @@ class Recursion:
         if kind == "A":
             return f"amp_task<{m}, R>(st, {{row}})"
         if kind == "S":
-            return "amp_task<1, R>(st, {row}, S0<R>)" if self.n == 4 else "amp_task<1, R>(st, {row})"
+            return "amp_task<1, R>(st, {row})"
         return "vec_task<R>(st, {row})"
 
     def stages(self):
@@ -415,8 +418,7 @@ class _Emit:
         """Vector index of an item for the thread's helicities (code)."""
         rec = self.rec
         g, sp = rec.items[key]
-        pos = f"S0<R> + {rec.base[key]}" if key[0] == "S" and rec.n == 4 else f"{rec.base[key]}"
-        a = f"{pos} + {self.offset(g)}" if g else pos
+        a = f"{rec.base[key]} + {self.offset(g)}" if g else f"{rec.base[key]}"
         if sp == 2:
             a += f" + ((s + 2 * (b0 + ib)) << {len(g)})"
         elif sp == 1:
@@ -799,7 +801,7 @@ def emit_recursion(n: int, tag: str) -> str:
     L.append(f"struct {tag}_rec {{")
     L.append(f"  static constexpr int N = {n}, NPAR = {n + 2}, NHEL = {1 << (n + 2)}, NCOL = {len(ws)};")
     L.append("  template <typename R>")
-    L.append(f"  static constexpr int NVEC = {rec.nvec}" + (f" + (sizeof(R) == 4 ? 0 : {rec.nlate});" if n == 4 else ";"))
+    L.append(f"  static constexpr int NVEC = {rec.nvec};")
     L.append(f"  static constexpr double IDEN = {iden}.0;")
     L.append(f"  static constexpr int CDEN = {cden}, NDIAG = {count_diagrams(n)}, NAMP = {len(build_plan(n).amps)};")
     L.append("  // colour numerators, flows in lexicographic order")
@@ -823,10 +825,6 @@ def emit_recursion(n: int, tag: str) -> str:
     L += body
     L.append("  }")
     if n <= 4:
-        if n == 4:
-            L.append(f"  // S over the {rec.nlate} vectors of A and C (FP32), or behind the others")
-            L.append("  template <typename R>")
-            L.append(f"  static constexpr int S0 = sizeof(R) == 4 ? 0 : {rec.nvec};")
         L.append(f"  static constexpr bool LATE = {'true' if late else 'false'};")
         L.append("  template <typename R, class ST>")
         L.append("  __device__ static __forceinline__ void late([[maybe_unused]] const ST& all, [[maybe_unused]] const int tid,")
