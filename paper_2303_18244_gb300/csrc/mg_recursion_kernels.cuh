@@ -37,6 +37,11 @@ struct RecShape {
   // per 65536.
   static constexpr int WARPS = P::N == 4 ? 12 : f32 ? 8 : 4;
   static constexpr int EV = WARPS * 32 / T;
+  // Five gluons in FP64: one event fills the shared memory, and its 4 warps leave
+  // the FP64 pipe idle for a quarter of the time.  As many helper threads share
+  // the lists of currents and half of the colour form.
+  static constexpr int HELP = P::N == 5 && !f32 ? T : 0;
+  static constexpr int MAXT = T * EV + HELP;
 };
 
 template <class P, typename R>
@@ -46,7 +51,7 @@ struct RecLayout {
   static constexpr size_t r128(size_t b) { return (b + 127) / 128 * 128; }
   static constexpr size_t mom_bytes = size_t(P::NPAR) * 4 * sizeof(double);  // per event
   static constexpr size_t red_off = 16;                                       // after the mbarrier: partial sums
-  static constexpr size_t mom_off = r128(red_off + RecShape<P, R>::WARPS * sizeof(double));
+  static constexpr size_t mom_off = r128(red_off + RecShape<P, R>::MAXT / 32 * sizeof(double));
   static constexpr size_t store_off = mom_off + r128(EV * mom_bytes);
   static constexpr size_t store_bytes = ST::stride;
   static constexpr size_t base_bytes = store_off + EV * store_bytes;
@@ -121,7 +126,7 @@ __device__ __forceinline__ double warp_scatter_sum(const double (&v)[N]) {
 template <int N>
 using Count = std::integral_constant<int, N>;
 
-// The event loop; blockDim.x = T * (events per tile).  body(store, e, valid)
+// The event loop; blockDim.x = T * (events per tile) + HELP.  body(store, e, valid)
 // runs with the currents complete; groups past the last event repeat it.
 template <class P, typename R, typename D, class BODY>
 __device__ __forceinline__ void rec_events(unsigned char* smem, const double* __restrict__ mom, long long nevt,
@@ -130,8 +135,9 @@ __device__ __forceinline__ void rec_events(unsigned char* smem, const double* __
   using ST = typename LY::ST;
   constexpr int T = LY::T;
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
-  const int tid = threadIdx.x, nt = blockDim.x, ge = tid / T;
-  const int per = nt / T;
+  constexpr bool help = RecShape<P, R>::HELP > 0;  // one event per tile
+  const int tid = threadIdx.x, nt = blockDim.x, ge = help ? 0 : tid / T;
+  const int per = help ? 1 : nt / T;
   const ST all(smem + LY::store_off), st = all.at(ge);
   const R kr[2] = {R(kp.v[0]), R(kp.v[1])};
   const long long step = (long long)gridDim.x * per;
@@ -331,15 +337,18 @@ __global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_
 // put(k, value), in the emitted order.
 template <class P, typename R, class ST, class GET, class PUT>
 __device__ __forceinline__ void rec_cta_flows(const ST& st, const KParams& kp, const GET& get, const PUT& put) {
-  const int gt = threadIdx.x % P::NHEL;
+  constexpr bool help = RecShape<P, R>::HELP > 0;
+  const int gt = threadIdx.x % P::NHEL, ge = help ? 0 : threadIdx.x / P::NHEL;
+  const bool main = !help || threadIdx.x < P::NHEL;
   const int hg = gt & ((1 << P::N) - 1), s = gt >> P::N & 1, b = gt >> (P::N + 1);
-  P::template closings<R, 1>(st, hg, s, b, [&](int, int k, cx<R> v) { put(k, v); });
+  if (main) P::template closings<R, 1>(st, hg, s, b, [&](int, int k, cx<R> v) { put(k, v); });
   __syncthreads();
   const R kr[2] = {R(kp.v[0]), R(kp.v[1])};
-  P::template late<R>(st.at(-(int)(threadIdx.x / P::NHEL)), kr, threadIdx.x, blockDim.x, blockDim.x / P::NHEL);
+  P::template late<R>(st.at(-ge), kr, threadIdx.x, blockDim.x, help ? 1 : blockDim.x / P::NHEL);
   __syncthreads();
-  P::template all_flows<R, 1>(
-      st, hg, s, b, [&](int, int k) { return get(k); }, [&](int, int k, cx<R> v) { put(k, v); });
+  if (main)
+    P::template all_flows<R, 1>(
+        st, hg, s, b, [&](int, int k) { return get(k); }, [&](int, int k, cx<R> v) { put(k, v); });
 }
 template <class P>
 __device__ __forceinline__ int rec_cta_helicity() {
@@ -350,11 +359,13 @@ __device__ __forceinline__ int rec_cta_helicity() {
 // Five gluons, one kernel; the thread's flows wait in local memory for the
 // colour form.
 template <class P, typename R, typename D, typename A, RecMode MODE>
-__global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_cta_kernel(LaunchArgs a) {
+__global__ void __launch_bounds__(RecShape<P, R>::MAXT, 1) rec_cta_kernel(LaunchArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   using LY = RecLayout<P, R>;
   constexpr int T = LY::T, NW = T / 32;
-  const int gt = threadIdx.x % T, ge = threadIdx.x / T, lane = threadIdx.x & 31, warp = gt >> 5;
+  constexpr bool help = RecShape<P, R>::HELP > 0;
+  const int gt = threadIdx.x % T, ge = help ? 0 : threadIdx.x / T, lane = threadIdx.x & 31, warp = gt >> 5;
+  const bool main = !help || threadIdx.x < T;
   const int hel = rec_cta_helicity<P>();
   bool good = false;
   if constexpr (MODE != REC_HELICITIES)
@@ -364,6 +375,41 @@ __global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_
     cx<R> fl[P::NCOL];
     rec_cta_flows<P, R>(
         st, a.kp, [&](int k) { return fl[k]; }, [&](int k, cx<R> v) { fl[k] = v; });
+    if constexpr (help && MODE == REC_SIGMA) {
+      // two of the four colour blocks go to the helper of the helicity, through
+      // the store's space once every thread has its flows
+      constexpr int NQ = P::NBLOCK;
+      static_assert(2 * NQ * T * sizeof(cx<R>) <= LY::store_bytes, "two blocks of every helicity");
+      cx<R>* x = reinterpret_cast<cx<R>*>(smem + LY::store_off) + gt;
+      cx<R> f[NQ];
+      __syncthreads();
+      if (main) {
+        P::template colour_blocks<R>(fl);
+        P::template colour_block<2, R>(fl, f);
+#pragma unroll
+        for (int q = 0; q < NQ; q++) x[q * T] = f[q];
+        P::template colour_block<3, R>(fl, f);
+#pragma unroll
+        for (int q = 0; q < NQ; q++) x[(NQ + q) * T] = f[q];
+      }
+      __syncthreads();
+      A v = A(0);
+#pragma unroll 1
+      for (int c = 0; c < 2; c++) {
+        if (!main) {
+#pragma unroll
+          for (int q = 0; q < NQ; q++) f[q] = x[(c * NQ + q) * T];
+        } else if (c == 0) {
+          P::template colour_block<0, R>(fl, f);
+        } else {
+          P::template colour_block<1, R>(fl, f);
+        }
+        v += (A)P::template block_value<R>(main ? c : 2 + c, f);
+      }
+      const A acc = rec_group_sum<2 * T>(good ? v : A(0), reinterpret_cast<A*>(smem + LY::red_off));
+      if (threadIdx.x == 0) a.out[e] = (double)(acc * A(norm));
+      return;
+    }
     // the choice's values take the store's space once every thread has its flows
     double* mh = reinterpret_cast<double*>(smem + LY::store_off + ge * LY::store_bytes);
     double* wp = mh + P::NHEL;       // [warp][flow]
@@ -377,22 +423,26 @@ __global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_
         for (int k = 0; k < 24; k++)
           sq[k] = good ? fl[k0 + k].re * fl[k0 + k].re + fl[k0 + k].im * fl[k0 + k].im : 0.0;
         const double w = warp_scatter_sum(sq);
-        if (lane < 24) wp[warp * P::NCOL + k0 + lane] = w;
+        if (main && lane < 24) wp[warp * P::NCOL + k0 + lane] = w;
       }
     }
-    A v;
-    if constexpr (MODE == REC_PAPER)
-      v = (A)P::colour_form_paper(fl);
-    else
-      v = (A)P::template colour_form<R>(fl);
+    A v = A(0);
+    if (main) {
+      if constexpr (MODE == REC_PAPER)
+        v = (A)P::colour_form_paper(fl);
+      else
+        v = (A)P::template colour_form<R>(fl);
+    }
+    valid = valid && main;
     if constexpr (MODE == REC_HELICITIES) {
       if (valid) a.out[e * P::NHEL + hel] = (double)v * norm;
     } else {
-      if constexpr (MODE == REC_SELECT) mh[hel] = (double)v;
+      if constexpr (MODE == REC_SELECT)
+        if (main) mh[hel] = (double)v;
       const A acc = rec_group_sum<T>(good ? v : A(0), reinterpret_cast<A*>(smem + LY::red_off));
       if (gt == 0 && valid) a.out[e] = (double)(acc * A(norm));
       if constexpr (MODE == REC_SELECT) {
-        if (gt < P::NCOL) {
+        if (main && gt < P::NCOL) {
           double w = 0.0;
           for (int q = 0; q < NW; q++) w += wp[q * P::NCOL + gt];
           wl[P::lex_flow(gt)] = w;
@@ -569,11 +619,11 @@ int launch_rec(const LaunchArgs& a) {
   }();
   static const cudaError_t attr = set_smem_attr(kernel, smem);
   if (attr != cudaSuccess) return -4;
-  static const int resident = rec_resident(kernel, LY::T * LY::EV, smem);
+  static const int resident = rec_resident(kernel, RecShape<P, R>::MAXT, smem);
   if (resident < 1) return -4;
   if (a.nevt <= 0) return 0;  // one-time set-up only
   const RecGrid g = rec_grid(a.nevt, resident, LY::EV);
-  kernel<<<g.grid, LY::T * g.per, smem, a.stream>>>(a);
+  kernel<<<g.grid, LY::T * g.per + RecShape<P, R>::HELP, smem, a.stream>>>(a);
   return cudaGetLastError() == cudaSuccess ? 0 : -4;
 }
 

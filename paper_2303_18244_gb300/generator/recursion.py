@@ -698,25 +698,30 @@ def _colour_form_looped(head, tag, n, K, ws) -> list[str]:
     tri = [M[chi][i][j] * (1 if i == j else 2) for chi in range(4) for i in range(no) for j in range(i, no)]
     head.insert(head.index(f"struct {tag}_rec {{"),
                 f"MG_REC_TABLE double {tag}_RECM[{len(tri)}] = {{" + ", ".join(str(x) for x in tri) + "};")
-    L = ["  // sum_ij KNUM_ij (Re J_i Re J_j + Im J_i Im J_j); |M|^2 colour sum = result / CDEN.",
-         "  // a[k]: flow k; overwritten by its block components",
+    L = [f"  // the flows' components in the four blocks of {no}, in their place", f"  static constexpr int NBLOCK = {no};",
          "  template <typename R>",
-         f"  __device__ static __forceinline__ R colour_form(cx<R> (&a)[{len(ws)}]) {{"]
+         f"  __device__ static __forceinline__ void colour_blocks(cx<R> (&a)[{len(ws)}]) {{"]
     for o in orbits:
         L.append(f"    {{ const cx<R> p0 = a[{o[0]}] + a[{o[1]}], m0 = a[{o[0]}] - a[{o[1]}], "
                  f"p1 = a[{o[2]}] + a[{o[3]}], m1 = a[{o[2]}] - a[{o[3]}];")
         L.append(f"      a[{o[0]}] = p0 + p1; a[{o[1]}] = m0 + m1; a[{o[2]}] = p0 - p1; a[{o[3]}] = m0 - m1; }}")
-    L.append("    R acc = R(0);")
-    size = no * (no + 1) // 2
-    for chi in range(4):
-        L.append("    {")
-        L.append(f"      const double* m = {tag}_RECM + {chi * size};")
-        L.append(f"      cx<R> f[{no}];")
-        L += [f"      f[{r}] = a[{o[chi]}];" for r, o in enumerate(orbits)]
-        L.append("      acc = acc + block_form<R>(m, f);")
-        L.append("    }")
-    L.append("    return R(0.25) * acc;")
     L.append("  }")
+    L += ["  // those of block CHI", "  template <int CHI, typename R>",
+          f"  __device__ static __forceinline__ void colour_block(const cx<R> (&a)[{len(ws)}], cx<R> (&f)[{no}]) {{"]
+    for chi in range(4):
+        L.append(f"    if constexpr (CHI == {chi}) {{ "
+                 + " ".join(f"f[{r}] = a[{o[chi]}];" for r, o in enumerate(orbits)) + " }")
+    L.append("  }")
+    L += ["  // sum_ij KNUM_ij (Re J_i Re J_j + Im J_i Im J_j); |M|^2 colour sum = result / CDEN.",
+          "  // a[k]: flow k; overwritten by its block components.  The sum of four blocks' values:",
+          "  template <typename R>",
+          f"  __device__ static __forceinline__ R block_value(int chi, const cx<R> (&f)[{no}]) {{",
+          f"    return R(0.25) * block_form<R>({tag}_RECM + {no * (no + 1) // 2} * chi, f);", "  }",
+          "  template <typename R>",
+          f"  __device__ static __forceinline__ R colour_form(cx<R> (&a)[{len(ws)}]) {{",
+          "    colour_blocks<R>(a);", "    R acc = R(0);", f"    cx<R> f[{no}];"]
+    L += [f"    colour_block<{chi}, R>(a, f); acc = acc + block_value<R>({chi}, f);" for chi in range(4)]
+    L += ["    return acc;", "  }"]
     B = ["  // one block: numerators M_ii and 2 M_ij (j > i) row by row",
          "  template <typename R>",
          f"  __device__ static __noinline__ R block_form(const double* __restrict__ m, const cx<R> (&f)[{no}]) {{",
