@@ -1,17 +1,17 @@
 // mg_colour_tc.cuh -- colour quadratic form on the 5th-generation tensor cores.
 //
 // Step A5 (paper Sect. 3: the "colour algebra" step run at reduced precision)
-// for a CTA of 128 events and one helicity:
-//     ME_h(e) = sum_ij Re/Im J_i(e) KNUM_ij Re/Im J_j(e)       (C = KNUM / CDEN)
-// is computed as D = A . KNUM with A = [128 events x K] (K = NCOL padded to a
-// multiple of 16) on the tensor cores, then a per-thread row dot J . D.
+// for the 128 helicities h of one event:
+//     ME_h = sum_ij Re/Im J_i(h) KNUM_ij Re/Im J_j(h)       (C = KNUM / CDEN)
+// is computed as D = A . KNUM with A = [128 helicities x K] (K = NCOL padded to
+// a multiple of 16) on the tensor cores, then a per-thread row dot J . D.
 //
 //   * KNUM holds small integers (|KNUM| <= 4096): exact in FP16.
 //   * A = s * J split into FP16 hi + lo (hi = fp16(sJ), lo = fp16(sJ - hi)),
-//     s a per-event power of two putting max|J| in [1, 2): the pair carries
+//     s a per-row power of two putting max|J| in [1, 2): the pair carries
 //     ~22 significant bits, and D = A_hi.KNUM + A_lo.KNUM accumulates in FP32.
 //   * Re and Im parts use two accumulators of N columns each in TMEM
-//     (cta_group::1, M = 128: row e of D lives in TMEM lane e).
+//     (cta_group::1, M = 128: row h of D lives in TMEM lane h).
 //   * One elected thread issues tcgen05.mma; completion is signalled on an
 //     mbarrier through tcgen05.commit; every wait is bounded.
 //

@@ -523,6 +523,12 @@ __global__ void __launch_bounds__(128, 2)
   for (long long e = blockIdx.x; e < nevt; e += gridDim.x) {
     const float2* row = J + e * (long long)(P::NCOL * NT) + tid;
     float fr[P::NCOL], fi[P::NCOL];
+    // the CTA's next rows on their way to L2 while this event is worked on (8229
+    // events 0.33 -> 0.285 ms)
+    if (tid == 0 && e + gridDim.x < nevt)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(row + (long long)gridDim.x * (P::NCOL * NT)),
+                   "r"((uint32_t)(P::NCOL * NT * sizeof(float2)))
+                   : "memory");
 #pragma unroll
     for (int k = 0; k < P::NCOL; k++) {
       const float2 v = __ldcs(row + k * NT);
@@ -642,11 +648,7 @@ int launch_rec_rows(const LaunchArgs& a) {
   static const int res2 = 2 * rec_sms();
   if (res1 < 1 || res2 < 1) return -4;
   if (a.nevt <= 0 || a.nhel <= 0) return 0;
-#ifdef MG_REC_SLICE
-  const size_t bytes = std::min<size_t>(rows_workspace_bytes(P::NCOL, a.nevt, a.nhel), (size_t)MG_REC_SLICE * P::NCOL * P::NHEL * 8);
-#else
   const size_t bytes = rows_workspace_bytes(P::NCOL, a.nevt, a.nhel);
-#endif
   const long long slice = (long long)(bytes / (sizeof(float2) * P::NCOL * P::NHEL));
   float2* J = nullptr;
   const cudaError_t e0 = a.pool ? cudaMallocFromPoolAsync(reinterpret_cast<void**>(&J), bytes, a.pool, a.stream)
