@@ -175,13 +175,16 @@ __global__ void __launch_bounds__(SCAN_T) tile_scan_kernel(long long* __restrict
 // launch 96.4 us.
 // Lane l takes words l*WPL .. of the tile, consecutive events; a tile with few
 // kept events writes them lane by lane, a fuller one word by word (coalesced).
+// bits and counts are still being written while this kernel's first blocks wait:
+// they are plain pointers, since const __restrict__ would promise that nothing
+// writes them during the kernel and so allow loads (also through the
+// non-coherent path) ahead of the wait.
 constexpr int WRITE_TILES = 16;
 constexpr long long SUM_TILES = 16384;
 
 template <bool SCANNED>
 __global__ void __launch_bounds__(UW_THREADS)
-    tile_write_kernel(const unsigned* __restrict__ bits, const long long* __restrict__ counts, long long ntiles,
-                      long long* __restrict__ n_acc, long long* __restrict__ idx_out) {
+    tile_write_kernel(unsigned* bits, long long* counts, long long ntiles, long long* n_acc, long long* idx_out) {
   constexpr int WPL = UW_WORDS / 32;               // words per lane
   constexpr int PER_WARP = WRITE_TILES / UW_WARPS;  // tiles per warp
   static_assert(UW_WORDS % 32 == 0 && WRITE_TILES <= 32, "whole warps of words, at most one tile count per lane");
@@ -298,7 +301,7 @@ extern "C" int mg_unweight(const double* w_dev, const double* r_dev, int64_t n, 
   cfg.attrs = &early;
   cfg.numAttrs = 1;
   cudaError_t e1 = cudaLaunchKernelEx(&cfg, ntiles > SUM_TILES ? tile_write_kernel<true> : tile_write_kernel<false>,
-                                      (const unsigned*)bits, (const long long*)counts, ntiles, acc, idx);
+                                      bits, counts, ntiles, acc, idx);
   const cudaError_t e3 = cudaGetLastError();
   if (e1 == cudaSuccess) e1 = e3;
   const cudaError_t e2 = cudaFreeAsync(counts, s);
