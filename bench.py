@@ -169,18 +169,15 @@ def load_flops(tag: str) -> dict:
         return json.load(f)[tag]
 
 
-def launches_per_sigma(proc: str, nevt: int, ngood: int) -> int:
+def launches_per_sigma(proc: str, nevt: int) -> int:
     """Kernel launches of one mixed mg_sigma call: one, except for gg -> t t~ g g g,
     whose two-phase path launches the flow and colour kernels once per slice
-    of the events, the slices sized to the workspace (at most 1 GiB: as many
-    rows of 120 complex FP32 flows of one helicity over the events, padded to
-    128, as fit, shared out as 128 helicities per event)."""
+    of the events (at most 8704: 120 complex FP32 flows of 128 helicities per
+    event in a workspace of at most 1 GiB, whole groups of 128 events)."""
     if proc != "ggttggg":
         return 1
-    per_hel = 120 * ((nevt + 127) // 128 * 128) * 8
-    hs = max(1, min(ngood, (1 << 30) // per_hel))
-    slice_events = hs * per_hel // (120 * 128 * 8)
-    return 2 * ((nevt + slice_events - 1) // slice_events)
+    most = (1 << 30) // (128 * 120 * 128 * 8) * 128
+    return 2 * ((nevt + most - 1) // most)
 
 
 def flops_per_event(fl: dict, ngood: int, recursion: bool) -> float:
@@ -473,7 +470,7 @@ def main():
                                             if hbm_peak else None,
                                             "bytes_per_event": "16 read (w, r) + 8 per kept index",
                                             "peak_source": "MEASURED_PEAKS.json hbm_gbs (copy)"}}},
-        "gpu_launches": args.steps * launches_per_sigma(args.proc, nevt, ngood),
+        "gpu_launches": args.steps * launches_per_sigma(args.proc, nevt),
         "clocks": clk,
     }
     if rank == 0 and not args.no_cpu_baseline:

@@ -118,14 +118,16 @@ int mg_good_helicities(mg_process* h, const double* momenta_dev, int64_t nevt, i
 /* ME per event on the device, stream-ordered and asynchronous:
  * me_out_dev[i] for momenta_dev[i], i < nevt.  nevt = 0 is a no-op.
  * The mixed path of g g > t t~ g g g runs in two phases through a workspace
- * of at most 1 GiB taken from the stream-ordered allocator (cudaMallocAsync)
- * and released on the same stream (capturable in a CUDA graph).
+ * of at most 1 GiB (larger calls run slice by slice) taken from the
+ * stream-ordered allocator and released on the same stream (capturable in a
+ * CUDA graph).  The cost of a call hardly depends on the helicity list: the
+ * gg processes and u u~ > t t~ g compute every helicity and sum the listed.
  * Errors: MG_ERR_ARG (NULL handle/pointer, nevt < 0, misaligned momenta),
  * MG_ERR_CUDA (launch failure, or no memory for that workspace). */
 int mg_sigma(mg_process* h, const double* momenta_dev, int64_t nevt, double* me_out_dev, void* stream);
 
 /* Device bytes that one mg_sigma call of nevt events takes from the
- * stream-ordered allocator with the handle's current helicity list: the
+ * stream-ordered allocator, whatever the handle's helicity list: the
  * two-phase workspace of the mixed g g > t t~ g g g path, 0 for every other
  * process and precision.  For memory planning (the serving loop's admission
  * counts it).  Errors: MG_ERR_ARG (NULL, nevt < 0). */

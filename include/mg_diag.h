@@ -38,8 +38,8 @@ typedef struct mg_process mg_process;
 
 /* One mg_sigma call (same arguments, same kernels) with CUDA events recorded
  * on the stream before the first kernel and after every kernel, for
- * processes whose ME call launches two kernels per slice of the good
- * helicities (the two-phase mixed g g > t t~ g g g path: colour flows to a
+ * processes whose ME call launches two kernels per slice of the
+ * events (the two-phase mixed g g > t t~ g g g path: colour flows to a
  * workspace, then the tensor-core colour form).  Waits for the stream.
  * *ms_first / *ms_second receive the summed durations of the first and
  * second kernel of every slice, *slices the number of slices.  Any output may

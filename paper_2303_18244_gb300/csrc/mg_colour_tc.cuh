@@ -211,21 +211,23 @@ struct LayoutRows {
 };
 
 // The stream-ordered workspace of one call: at most ROWS_WORKSPACE bytes of
-// flows (FP32 complex).
+// flows (FP32 complex).  The flow kernel writes every helicity of an event,
+// whatever the list, so the workspace is a number of events, the same for every
+// list: the call's, padded to 128, or as many as fit (8704 of 120 flows and 128
+// helicities); larger calls run slice by slice.  When it was shared out by the
+// listed helicities, 256 events with 94 of 128 listed took two slices and 117
+// us instead of 69, and from 1.1 M events on it grew past the bound.
 constexpr size_t ROWS_WORKSPACE = size_t(1) << 30;
 
-// Its size, in rows of one helicity over the events padded to 128: as many
-// helicities as fit ROWS_WORKSPACE (at least one, at most nhel).
-inline long long rows_ld(long long nevt) { return (nevt + 127) / 128 * 128; }
-inline long long rows_slice(int ncol, long long nevt, int nhel) {
-  const size_t per_hel = (size_t)ncol * (size_t)rows_ld(nevt) * sizeof(float2);
-  const long long hs = (long long)(ROWS_WORKSPACE / per_hel);
-  return hs < 1 ? 1 : (hs > nhel ? nhel : hs);
+// events of one slice (nhel: all helicities of the process)
+inline long long rows_slice(int ncol, int nhel, long long nevt) {
+  const size_t per128 = 128 * size_t(ncol) * size_t(nhel) * sizeof(float2);
+  const long long most = (long long)(ROWS_WORKSPACE / per128) * 128, all = (nevt + 127) / 128 * 128;
+  return all < most ? all : most;
 }
 // bytes one two-phase launch takes from the stream-ordered allocator
-inline size_t rows_workspace_bytes(int ncol, long long nevt, int nhel) {
-  if (nevt <= 0 || nhel <= 0) return 0;
-  return (size_t)rows_slice(ncol, nevt, nhel) * (size_t)ncol * (size_t)rows_ld(nevt) * sizeof(float2);
+inline size_t rows_workspace_bytes(int ncol, int nhel, long long nevt) {
+  return nevt <= 0 ? 0 : size_t(rows_slice(ncol, nhel, nevt)) * size_t(ncol) * size_t(nhel) * sizeof(float2);
 }
 
 }  // namespace mg

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <mutex>
+#include <new>
 
 #include "mg.h"
 #include "mg_colour_tc.cuh"
@@ -162,9 +163,11 @@ extern "C" int mg_diag_sigma_phases(mg_process* h, const double* momenta_dev, in
   int prev = -1;
   cudaGetDevice(&prev);
   if (prev != h->device) cudaSetDevice(h->device);
-  mg::PhaseMarks marks;
-  int made = 0, rc = MG_OK;
-  for (; made < mg::PhaseMarks::MAX; made++)
+  // a mark before the first kernel and after every kernel of every slice
+  const int64_t slice = mg::rows_slice(h->d->ncol, h->d->nhel, nevt), most = 1 + 2 * ((nevt + slice - 1) / slice);
+  mg::PhaseMarks marks{most < (1 << 20) ? new (std::nothrow) cudaEvent_t[most] : nullptr, (int)most};
+  int made = 0, rc = marks.ev ? MG_OK : MG_ERR_NOMEM;
+  for (; marks.ev && made < marks.max; made++)
     if (cudaEventCreate(&marks.ev[made]) != cudaSuccess) {
       rc = MG_ERR_CUDA;
       break;
@@ -189,6 +192,7 @@ extern "C" int mg_diag_sigma_phases(mg_process* h, const double* momenta_dev, in
     }
   }
   for (int i = 0; i < made; i++) cudaEventDestroy(marks.ev[i]);
+  delete[] marks.ev;
   if (prev >= 0 && prev != h->device) cudaSetDevice(prev);
   if (rc != MG_OK) return rc;
   if (ms_first) *ms_first = t1;

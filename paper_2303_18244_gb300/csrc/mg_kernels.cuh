@@ -372,11 +372,10 @@ struct LaunchArgs {
 };
 
 struct PhaseMarks {
-  static constexpr int MAX = 257;
-  cudaEvent_t ev[MAX];
-  int n = 0;
+  cudaEvent_t* ev;  // room for max marks
+  int max, n = 0;
   void mark(cudaStream_t s) {
-    if (n < MAX) cudaEventRecord(ev[n++], s);
+    if (n < max) cudaEventRecord(ev[n++], s);
   }
 };
 

@@ -633,8 +633,7 @@ int launch_rec(const LaunchArgs& a) {
   return cudaGetLastError() == cudaSuccess ? 0 : -4;
 }
 
-// The two phases over slices of the events that fit the workspace (sized by
-// rows_workspace_bytes: at most 1 GiB, and never less than one event).
+// The two phases over slices of the events that fit the workspace (rows_slice).
 template <class P>
 int launch_rec_rows(const LaunchArgs& a) {
   using LY = RecLayout<P, float>;
@@ -648,8 +647,8 @@ int launch_rec_rows(const LaunchArgs& a) {
   static const int res2 = 2 * rec_sms();
   if (res1 < 1 || res2 < 1) return -4;
   if (a.nevt <= 0 || a.nhel <= 0) return 0;
-  const size_t bytes = rows_workspace_bytes(P::NCOL, a.nevt, a.nhel);
-  const long long slice = (long long)(bytes / (sizeof(float2) * P::NCOL * P::NHEL));
+  const size_t bytes = rows_workspace_bytes(P::NCOL, P::NHEL, a.nevt);
+  const long long slice = rows_slice(P::NCOL, P::NHEL, a.nevt);
   float2* J = nullptr;
   const cudaError_t e0 = a.pool ? cudaMallocFromPoolAsync(reinterpret_cast<void**>(&J), bytes, a.pool, a.stream)
                                 : cudaMallocAsync(reinterpret_cast<void**>(&J), bytes, a.stream);

@@ -250,15 +250,14 @@ int mg_launch_sigma(mg_process* h, const double* mom, int64_t nevt, double* me, 
   return mg_launch_sigma_locked(h, mom, nevt, me, stream);
 }
 
-int64_t mg_workspace_bytes_locked(const mg_process* h, int64_t nevt) {
+int64_t mg_workspace_bytes(const mg_process* h, int64_t nevt) {
   if (h->par.precision != MG_MIXED || !h->d->rows_mixed) return 0;
-  return (int64_t)mg::rows_workspace_bytes(h->d->ncol, nevt, h->n_good);
+  return (int64_t)mg::rows_workspace_bytes(h->d->ncol, h->d->nhel, nevt);
 }
 
 extern "C" int mg_sigma_workspace_bytes(mg_process* h, int64_t nevt, int64_t* bytes_out) {
   if (!h || nevt < 0 || !bytes_out) return MG_ERR_ARG;
-  std::lock_guard<std::mutex> lk(h->lock);
-  *bytes_out = mg_workspace_bytes_locked(h, nevt);
+  *bytes_out = mg_workspace_bytes(h, nevt);
   return MG_OK;
 }
 

@@ -39,5 +39,5 @@ int mg_launch_sigma(mg_process* h, const double* mom, int64_t nevt, double* me, 
 // records an event before and after each kernel of a multi-kernel launch
 int mg_launch_sigma_locked(mg_process* h, const double* mom, int64_t nevt, double* me, cudaStream_t stream,
                            mg::PhaseMarks* marks = nullptr);
-// stream-ordered workspace bytes of one launch of nevt events (h->lock held)
-int64_t mg_workspace_bytes_locked(const mg_process* h, int64_t nevt);
+// stream-ordered workspace bytes of one launch of nevt events
+int64_t mg_workspace_bytes(const mg_process* h, int64_t nevt);

@@ -132,12 +132,7 @@ static int64_t bucket_for(const mg_server_cfg& c, int64_t n) {
 // device bytes a chunk holds while in flight: momenta and results of its
 // bucket, and the workspace of its launch
 static int64_t chunk_bytes(mg_process* h, int64_t bucket) {
-  int64_t ws;
-  {
-    std::lock_guard<std::mutex> lk(h->lock);
-    ws = mg_workspace_bytes_locked(h, bucket);
-  }
-  return bucket * (h->d->npar * 32 + 8) + ws;
+  return bucket * (h->d->npar * 32 + 8) + mg_workspace_bytes(h, bucket);
 }
 
 void mg_server::finish_chunk(Request* r, int rc) {
