@@ -41,23 +41,31 @@ struct PSArgs {
   double sqrt_s;
   uint64_t seed;
   long long first_event, nevt;
-  double mass;  // of the first two final states
-  double mu2;   // (mass / sqrt_s)^2
+  double unit;  // the power of two with sqrt_s / unit in [1, 2)
+  double rs;    // sqrt_s / unit, exact
+  double mass;  // of the first two final states / unit, exact
   double xi0;   // sqrt(1 - (sum of the masses / sqrt_s)^2): start of the scale
 };
 
 // One event per thread, everything in registers (NF final states, a template
 // parameter).  The FP64 pipe bounds it (16 cycles per warp instruction and
 // SM): about 530 FP64 instructions per event for NF = 4.  The map works on
-// momenta in units of the generated mass M and solves for X = (scale) /
-// sqrt_s in f(X) = sum_j sqrt(mu_j^2 + X^2 |p_j|^2) - 1 = 0:
-//   - Newton in FP32 first, which leaves about 1e-7;
+// momenta in units of the generated mass M; their scale x onto the mass shells
+// solves f(x) = sum_j sqrt(m_j^2 + x^2 |p_j|^2) - sqrt_s = 0:
+//   - Newton in FP32 first, which leaves about 1e-7 (NF > 2; for two equal
+//     masses the start is the solution up to the rounding of the map);
 //   - then FP64 steps with the FP32 derivative, each of which gains those
-//     seven digits again; a step below 1e-9 of X leaves less than the rounding
+//     seven digits again; a step below 1e-9 of x leaves less than the rounding
 //     of f, so two steps are usual (at most 60).
-// Newton in FP64 alone, until a step fell below 1e-16 of X, took as many
-// iterations as the slowest lane of the warp needed to meet a bound below the
-// rounding of f (up to all 60): 524288 events of NF = 4 5.66 ms.
+// Masses, sqrt_s and x are in units of a power of two, so that nothing is
+// rounded before sqrt_s and the masses cancel in f: in units of sqrt_s itself
+// the gluons lost digits near threshold (energies off by 1e-8 at sqrt_s = 2 m_t
+// (1 + 1e-9), 1e-5 at 1e-12; by 1e-10 and 1e-13 now, five final states).
+// Against 113-bit values, mean error of a component over its energy at four
+// final states: 9.0e-17 (9.1e-17 in units of sqrt_s, 11.9e-17 with Newton in
+// FP64 alone, until a step fell below 1e-16 of x: as many iterations as the
+// slowest lane of the warp needed to meet a bound below the rounding of f, up to
+// all 60; 524288 events 5.66 ms).
 template <int NF, bool ALIGNED>
 __global__ void __launch_bounds__(128) rambo_kernel(PSArgs a, double* __restrict__ out) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -91,7 +99,7 @@ __global__ void __launch_bounds__(128) rambo_kernel(PSArgs a, double* __restrict
   const double im = 1.0 / M;
   const double b[3] = {-Q[1] * im, -Q[2] * im, -Q[3] * im};
   const double aa = 1.0 / ::fma(Q[0], im, 1.0);
-  // 3-momenta in the centre-of-mass frame, in units of M / sqrt_s
+  // 3-momenta in the centre-of-mass frame, in units of M
   double R3[3] = {0, 0, 0};
 #pragma unroll
   for (int j = 0; j < NF; j++) {
@@ -119,44 +127,48 @@ __global__ void __launch_bounds__(128) rambo_kernel(PSArgs a, double* __restrict
     }
   }
   // common scale onto the mass shells
-  const double x0 = a.xi0 * im;
-  const float mu2f = (float)a.mu2, Sf = (float)S;
-  float xf = (float)x0, dinv = 0.f;
+  const double x0 = a.xi0 * im * a.rs, m2 = a.mass * a.mass;
+  const float Sf = (float)S;
+  double x = x0;
+  if constexpr (NF > 2) {
+    const float m2f = (float)m2, rsf = (float)a.rs;
+    float xf = (float)x0, dinv = 0.f;
 #pragma unroll 1
-  for (int it = 0; it < 6; it++) {
-    float f = fmaf(xf, Sf, -1.f), df = Sf;
+    for (int it = 0; it < 6; it++) {
+      float f = fmaf(xf, Sf, -rsf), df = Sf;
 #pragma unroll
-    for (int j = 0; j < 2; j++) {
-      const float r = rsqrtf(fmaf(xf * xf, p2f[j], mu2f));
-      f = fmaf(fmaf(xf * xf, p2f[j], mu2f), r, f);
-      df = fmaf(xf * p2f[j], r, df);
+      for (int j = 0; j < 2; j++) {
+        const float r = rsqrtf(fmaf(xf * xf, p2f[j], m2f));
+        f = fmaf(fmaf(xf * xf, p2f[j], m2f), r, f);
+        df = fmaf(xf * p2f[j], r, df);
+      }
+      dinv = 1.f / df;
+      xf = fmaf(-f, dinv, xf);
     }
-    dinv = 1.f / df;
-    xf = fmaf(-f, dinv, xf);
+    // else FP32 did not converge
+    if (xf > 0.f && xf < 1e30f && dinv > 0.f && dinv < 1e30f) x = (double)xf;
   }
-  double X = (double)xf;
-  if (!(xf > 0.f) || !(xf < 1e30f) || !(dinv > 0.f) || !(dinv < 1e30f)) X = x0;  // FP32 did not converge
 #pragma unroll 1
   for (int it = 0; it < 60; it++) {
-    double f = ::fma(X, S, -1.0), df = S;
-    const double X2 = X * X;
-    const float Xf = (float)X;
+    double e[2], df;
+    const double x2 = x * x;
+    const float xf = (float)x;
     float dm = Sf;
 #pragma unroll
     for (int j = 0; j < 2; j++) {
-      const double e = sqrt(::fma(X2, p2[j], a.mu2));
-      f += e;
-      dm = fmaf(Xf * p2f[j], 1.f / (float)e, dm);
+      e[j] = sqrt(::fma(x2, p2[j], m2));
+      dm = fmaf(xf * p2f[j], 1.f / (float)e[j], dm);
     }
+    const double f = ::fma(x, S, (e[0] - a.rs) + e[1]);
     df = (double)(1.f / dm);
     if (!(dm > 1e-30f) || !(dm < 1e30f)) {  // outside the FP32 range: the derivative in FP64
       df = S;
-      for (int j = 0; j < 2; j++) df += X * p2[j] / sqrt(::fma(X2, p2[j], a.mu2));
+      for (int j = 0; j < 2; j++) df += x * p2[j] / sqrt(::fma(x2, p2[j], m2));
       df = 1.0 / df;
     }
     const double step = f * df;
-    X -= step;
-    if (fabs(step) <= 1e-9 * fabs(X)) break;
+    x -= step;
+    if (fabs(step) <= 1e-9 * fabs(x)) break;
   }
   double* o = out + i * (long long)(NF + 2) * 4;
   auto put = [&](int slot, double e, double x, double y, double z) {
@@ -171,13 +183,14 @@ __global__ void __launch_bounds__(128) rambo_kernel(PSArgs a, double* __restrict
       t[3] = z;
     }
   };
-  const double E = 0.5 * a.sqrt_s, scale = X * a.sqrt_s, m2 = a.mass * a.mass;
+  const double E = 0.5 * a.sqrt_s, scale = x * a.unit;
   put(0, E, 0.0, 0.0, E);
   put(1, E, 0.0, 0.0, -E);
 #pragma unroll
   for (int j = 0; j < NF; j++)
-    put(2 + j, j < 2 ? sqrt(::fma(scale * scale, p2[j], m2)) : scale * root[j], scale * q[j][1], scale * q[j][2],
-        scale * q[j][3]);
+    // two equal masses: half of sqrt_s each
+    put(2 + j, NF == 2 ? E : (j < 2 ? a.unit * sqrt(::fma(x * x, p2[j], m2)) : scale * root[j]), scale * q[j][1],
+        scale * q[j][2], scale * q[j][3]);
 }
 
 template <int NF>
@@ -205,10 +218,12 @@ extern "C" int mg_rambo(const mg_process* h, double sqrt_s, uint64_t seed, int64
   if (nf < 2 || nf > 5) return MG_ERR_ARG;
   // final-state masses: the top pair of g g -> t t~ (+ gluons); massless leptons
   const bool tops = std::strcmp(h->d->tag, "eemumu") != 0;
-  a.mass = tops ? h->par.mt : 0.0;
-  if (2.0 * a.mass >= sqrt_s) return MG_ERR_ARG;
-  a.mu2 = (a.mass / sqrt_s) * (a.mass / sqrt_s);
-  a.xi0 = std::sqrt(1.0 - (2.0 * a.mass / sqrt_s) * (2.0 * a.mass / sqrt_s));
+  const double mass = tops ? h->par.mt : 0.0;
+  if (2.0 * mass >= sqrt_s) return MG_ERR_ARG;
+  a.unit = std::ldexp(1.0, std::ilogb(sqrt_s));
+  a.rs = sqrt_s / a.unit;
+  a.mass = mass / a.unit;
+  a.xi0 = std::sqrt(1.0 - (2.0 * mass / sqrt_s) * (2.0 * mass / sqrt_s));
   int prev = -1, dev = h->device;
   cudaGetDevice(&prev);
   if (prev != dev) cudaSetDevice(dev);
