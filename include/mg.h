@@ -57,8 +57,7 @@ extern "C" {
 #define MG_FP64 0   /* every step in FP64                                        */
 #define MG_MIXED 1  /* FP32 wavefunctions/amplitudes, FP64 propagator denominators,
                        FP32 colour sum (g g > t t~ g g g: FP16 hi+lo on the tensor
-                       cores, FP32 accumulation), helicity sum in FP64 or as FP32
-                       pairs with exact rounding errors                           */
+                       cores, FP32 accumulation), FP64 helicity sum              */
 #define MG_MIXED_PAPER 2 /* the paper's "mixed" (Sect. 3): Feynman diagrams in FP64,
                        colour algebra in FP32 on CUDA cores, FP64 helicity sum    */
 #define MG_FLOAT 3  /* the paper's "float" (Sect. 3): every step in FP32, the

@@ -199,9 +199,11 @@ __device__ __forceinline__ unsigned good_mask(const int* __restrict__ hels, int 
 // computed once per helicity combination of its own legs: a third of the
 // instructions of sigma_kernel, which evaluates every helicity by itself.
 // CTAS: CTAs per SM the registers are sized for.  Measured (us): g g -> t t~,
-// mixed, 524288 events, 2 / 3 / 4 CTAs 147 / 129 / 148 (sigma_kernel 192; FP64
-// set-up half of the FP64 pipe's time); u u~ -> t t~ g, all-float, 262147
-// events, 2 / 3 CTAs 85 / 96 (sigma_kernel 176), mixed 155 / 171.
+// mixed, 524288 events, 2 / 3 / 4 CTAs 147 / 129 / 148 (sigma_kernel 192); u u~ -> t t~ g, all-float, 262147
+// events, 2 / 3 CTAs 85 / 96 (sigma_kernel 176), mixed 155 / 171.  The helicity
+// sum stays in FP64: as an FP32 pair, which GB300 adds faster (its FP64 pipe
+// takes 16 cycles per warp instruction; g g -> t t~ mixed 129 -> 123), it holds
+// 1e-14 instead of 1e-16 and overflows where the terms do not.
 template <class P, typename R, typename D, typename A, int NT, int CTAS>
 __global__ void __launch_bounds__(NT, CTAS) sigma_thread_kernel(const double* __restrict__ mom, long long nevt,
                                                           double* __restrict__ me, const int* __restrict__ hels,

@@ -76,33 +76,6 @@ __device__ __forceinline__ A rec_group_sum(A v, A* red) {
   return v;
 }
 
-template <int T>
-__device__ __forceinline__ double rec_group_sum(PairSum v, void* red) {
-#pragma unroll
-  for (int o = (T < 32 ? T : 32) / 2; o > 0; o >>= 1) {
-    PairSum x;
-    x.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
-    x.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
-    v.add(x);
-  }
-  if constexpr (T > 32) {
-    constexpr int NW = T / 32;
-    PairSum* slot = static_cast<PairSum*>(red);
-    const int warp = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) slot[warp] = v;
-    __syncthreads();
-    v = PairSum{};
-#pragma unroll
-    for (int w = 0; w < NW; w++) v.add(slot[warp / NW * NW + w]);
-    __syncthreads();
-  }
-  return v.value();
-}
-template <int T, typename A>
-__device__ __forceinline__ A rec_group_sum(const PlainSum<A>& v, void* red) {
-  return rec_group_sum<T>(v.v, static_cast<A*>(red));
-}
-
 // reduce-scatter of N <= 32 values over a warp: lane k < N returns the sum
 // over the lanes of their v[k] (31 additions instead of 5 per value)
 template <int N>
@@ -263,7 +236,7 @@ __global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_
   double* wk = mh + P::NHEL;
   rec_events<P, R, D>(smem, a.mom, a.nevt, a.kp, a.status, [&](const auto& st, long long e, bool valid) {
     constexpr double norm = 1.0 / (P::IDEN * P::CDEN);
-    HelicitySum<R, A> part;
+    A part = A(0);
     [[maybe_unused]] double w = 0.0;
     const auto close = [&](const int b0) {
       cx<R> f[NB][P::NCOL];
@@ -285,7 +258,7 @@ __global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_
         if constexpr (MODE == REC_HELICITIES) {
           if (valid) a.out[e * P::NHEL + P::helicity(hg, s, b0 + ib)] = (double)v * norm;
         } else if (in) {
-          part.add(v);
+          part += (A)v;
         }
         if constexpr (MODE == REC_SELECT) {
           static_assert(P::NCOL <= (T < 32 ? T : 32), "lane k of the group sums flow k");
@@ -313,7 +286,7 @@ __global__ void __launch_bounds__(RecShape<P, R>::T* RecShape<P, R>::EV, 1) rec_
       for (int b0 = 0; b0 < 2; b0 += NB) close(b0);
     }
     if constexpr (MODE != REC_HELICITIES) {
-      const A acc = rec_group_sum<T>(part, smem + LY::red_off);
+      const A acc = rec_group_sum<T>(part, reinterpret_cast<A*>(smem + LY::red_off));
       if (gt == 0 && valid) a.out[e] = (double)(acc * A(norm));
       if constexpr (MODE == REC_SELECT) {
         const int lane = gt & 31;

@@ -342,34 +342,6 @@ __host__ __device__ __forceinline__ void two_sum(D a, D b, D& s, D& e) {
   const D bb = s - a;
   e = (a - (s - bb)) + (b - bb);
 }
-// Sum of FP32 values in FP64, or in the mixed mode as an FP32 pair whose low
-// part collects the exact rounding errors of the high part: 1e-14 or better,
-// far below the FP32 values' own rounding, and no FP64 instruction per value
-// (GB300's FP64 pipe takes 16 cycles per warp instruction and SM; the sums
-// over the helicities were a quarter of the mixed kernels' use of it).
-template <typename A>
-struct PlainSum {
-  A v = A(0);
-  __device__ __forceinline__ void add(A x) { v += x; }
-  __device__ __forceinline__ A value() const { return v; }
-};
-struct PairSum {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    float e;
-    two_sum(hi, x, hi, e);
-    lo += e;
-  }
-  __device__ __forceinline__ void add(const PairSum& o) {
-    add(o.hi);
-    lo += o.lo;
-  }
-  // an infinite or NaN sum has no rounding error to add
-  __device__ __forceinline__ double value() const { return lo == lo ? (double)hi + (double)lo : (double)hi; }
-};
-template <typename R, typename A>
-using HelicitySum = typename std::conditional<sizeof(R) == 4 && sizeof(A) == 8, PairSum, PlainSum<A>>::type;
-
 template <typename R, typename D, int N>
 __device__ __forceinline__ D inv_mass2(const D* const (&v)[N], const D (&s)[N], D m2) {
   if constexpr (sizeof(R) == 8 && sizeof(D) == 8) {

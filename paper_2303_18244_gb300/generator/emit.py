@@ -1109,7 +1109,7 @@ def _uuttg_thread_sum(dec) -> list[str]:
          "    kb.v[mu] = R(2) * kx[mu] + ky[mu];",
          "    kd.v[mu] = kx[mu] - ky[mu];",
          "  }",
-         "  HelicitySum<R, A> acc;",
+         "  A acc = A(0);",
          "#pragma unroll 1",
          "  for (int e = 0; e < 2; e++) {  // gluon helicity 2 e - 1",
          "    const V4<R> eps = ext_vector<R>(e1, e2, R(2 * e - 1), true);",
@@ -1155,8 +1155,8 @@ def _uuttg_thread_sum(dec) -> list[str]:
         L.append(f"          jamp[{m}] = " + " + ".join(terms) + ";")
     L += ["          const R v = colour_quadratic<R>(jamp, 1);",
           "          const int hel = (h << 4) | ((1 - h) << 3) | (s << 2) | (b << 1) | e;",
-          "          if (good >> hel & 1u) acc.add(v);",
-          "        }", "      }", "    }", "  }", "  return acc.value();",
+          "          if (good >> hel & 1u) acc += (A)v;",
+          "        }", "      }", "    }", "  }", "  return acc;",
           "#undef MOM", "#undef ING", "#undef EV", "}"]
     return L
 

@@ -600,7 +600,7 @@ def _thread_sum(rec: Recursion) -> list[str]:
          "    using namespace rec;",
          f"    const RegStore<R, {rec.n}, {rec.nvec}> st{{}};",
          "    const R kr[2] = {R(kp[0]), R(kp[1])};",
-         "    setup_thread<" + "P_SELF" + ", R, D>(st, p, kp, kr);", "    HelicitySum<R, A> acc;"]
+         "    setup_thread<" + "P_SELF" + ", R, D>(st, p, kp, kr);", "    A acc = A(0);"]
     calls: dict = {None: [], 0: [], 1: []}
     for stage, keys in rec.tasks.items():
         for key in keys:
@@ -617,8 +617,8 @@ def _thread_sum(rec: Recursion) -> list[str]:
             for hg in range(1 << rec.n):
                 L.append(f"    {{ cx<R> a[1][2]; flows_open<R, 1>(st, {hg}, {s}, {b}, a); flows_block<R, 1>(st, {hg}, {s}, {b}, a);")
                 L.append("      const R v = colour_form<R>(a[0]);")
-                L.append(f"      if (good >> helicity({hg}, {s}, {b}) & 1u) acc.add(v); }}")
-    L += ["    return acc.value();", "  }"]
+                L.append(f"      if (good >> helicity({hg}, {s}, {b}) & 1u) acc += (A)v; }}")
+    L += ["    return acc;", "  }"]
     return L
 
 
