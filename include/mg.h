@@ -117,10 +117,12 @@ int mg_good_helicities(mg_process* h, const double* momenta_dev, int64_t nevt, i
 /* ME per event on the device, stream-ordered and asynchronous:
  * me_out_dev[i] for momenta_dev[i], i < nevt.  nevt = 0 is a no-op.
  * The mixed path of g g > t t~ g g g runs in two phases through a workspace
- * of at most 1 GiB (larger calls run slice by slice) taken from the
- * stream-ordered allocator and released on the same stream (capturable in a
- * CUDA graph).  The cost of a call hardly depends on the helicity list: the
- * gg processes and u u~ > t t~ g compute every helicity and sum the listed.
+ * of at most 1 GiB (larger calls run slice by slice), allocated and freed in
+ * stream order (capturable in a CUDA graph) from a memory pool that the
+ * handles of this path share per device.  The pool keeps up to 1 GiB between
+ * calls and gives it back when the last of these handles is destroyed.
+ * The cost of a call hardly depends on the helicity list: the gg processes and
+ * u u~ > t t~ g compute every helicity and sum the listed ones.
  * Errors: MG_ERR_ARG (NULL handle/pointer, nevt < 0, misaligned momenta),
  * MG_ERR_CUDA (launch failure, or no memory for that workspace). */
 int mg_sigma(mg_process* h, const double* momenta_dev, int64_t nevt, double* me_out_dev, void* stream);

@@ -366,7 +366,7 @@ struct LaunchArgs {
   int* hel_out;
   int* col_out;
   double* colw_out;
-  // memory pool of the handle for the two-phase workspace (null: the device's)
+  // memory pool of the two-phase workspace (null: the device's)
   cudaMemPool_t pool;
   // diagnostics (may be null): events recorded on the stream before the first
   // and after every kernel of a multi-kernel launch

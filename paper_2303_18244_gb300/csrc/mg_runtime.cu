@@ -46,6 +46,51 @@ struct DeviceGuard {
   }
 };
 
+// The pool of the two-phase workspaces on a device, shared by its handles.  It
+// keeps up to one workspace (1 GiB) between calls, however many handles there
+// are, and goes with the last of them: the device's default pool returns its
+// memory at every synchronisation, and mapping 1 GiB again took 0.8 ms of a 3.0
+// ms call (8229 events).  Stream-ordered, so concurrent calls on several
+// streams get workspaces of their own.
+struct WorkspacePool {
+  cudaMemPool_t pool = nullptr;
+  int users = 0;
+};
+constexpr int MAX_DEVICES = 64;
+std::mutex pools_lock;
+WorkspacePool pools[MAX_DEVICES];
+
+cudaMemPool_t acquire_pool(int device) {
+  if (device < 0 || device >= MAX_DEVICES) return nullptr;
+  std::lock_guard<std::mutex> lk(pools_lock);
+  WorkspacePool& w = pools[device];
+  if (!w.pool) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    uint64_t keep = mg::ROWS_WORKSPACE;
+    cudaMemPool_t made = nullptr;
+    if (cudaMemPoolCreate(&made, &props) != cudaSuccess) return nullptr;
+    if (cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaMemPoolDestroy(made);
+      return nullptr;
+    }
+    w.pool = made;
+  }
+  w.users++;
+  return w.pool;
+}
+
+void release_pool(int device) {
+  std::lock_guard<std::mutex> lk(pools_lock);
+  WorkspacePool& w = pools[device];
+  if (--w.users > 0) return;
+  cudaMemPoolDestroy(w.pool);
+  w.pool = nullptr;
+}
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace
@@ -169,19 +214,8 @@ extern "C" int mg_process_create(const char* proc, const mg_params* p, mg_proces
     }
   }
   if (p->precision == MG_MIXED && d->rows_mixed) {
-    // The workspace comes from a pool of the handle's own that keeps up to one
-    // workspace between calls: the device's default pool returns its memory at
-    // every synchronisation, and mapping 1 GiB again took 0.8 ms of a 3.0 ms
-    // call (8229 events).  Stream-ordered, so concurrent calls on several
-    // streams get workspaces of their own; released with the handle.
-    cudaMemPoolProps props{};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.handleTypes = cudaMemHandleTypeNone;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = h->device;
-    uint64_t keep = mg::ROWS_WORKSPACE;
-    if (cudaMemPoolCreate(&h->pool, &props) != cudaSuccess ||
-        cudaMemPoolSetAttribute(h->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    h->pool = acquire_pool(h->device);
+    if (!h->pool) {
       mg_process_destroy(h);
       return MG_ERR_NOMEM;
     }
@@ -209,7 +243,7 @@ extern "C" void mg_process_destroy(mg_process* h) {
   cudaFree(h->d_ctile);
   cudaFree(h->d_mom);
   cudaFree(h->d_me);
-  if (h->pool) cudaMemPoolDestroy(h->pool);
+  if (h->pool) release_pool(h->device);
   delete h;
 }
 

@@ -23,7 +23,7 @@ struct mg_process {
   std::vector<uint8_t> mask;
   unsigned* d_status = nullptr;     // device status word (bounded-wait timeouts)
   void* d_ctile = nullptr;          // FP16 colour-matrix operand tile (mixed, tensor cores)
-  cudaMemPool_t pool = nullptr;     // two-phase workspace (rows_mixed), see mg_process_create
+  cudaMemPool_t pool = nullptr;     // two-phase workspace (rows_mixed), shared by the device's handles
   std::mutex lock;
   // workspace of mg_sigma_host
   std::mutex ws_lock;
