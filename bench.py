@@ -55,11 +55,11 @@ WORKLOADS = {
 }
 METRIC = "gg→tt̄gg MEs/s on 1 GB300, FP64 vs mixed (≤1e-5 rel err); serve p50/p99 ms"
 L2_FLUSH_BYTES = 256 << 20
-# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of the mixed
-# kernel from one ncu capture (rec_kernel of g g -> t t~ g g, mixed,
-# 65536 events, one launch): workload -> (events captured, bytes, digest of
-# the kernel sources that it holds for); scaled to a launch by its events (the
-# traffic is per event: momenta in, |M|^2 out).  Reported as null once the
+# DRAM reads (dram__bytes_read.sum) of the mixed kernel from one ncu capture
+# (rec_kernel of g g -> t t~ g g, mixed, 65536 events, one launch): workload ->
+# (events captured, bytes, digest of the kernel sources that were captured);
+# scaled to a launch by its events.  The writes are counted, 8 bytes per event:
+# the results of a capture of this size stay in L2.  Reported as null once the
 # sources differ from the captured ones (kernel_digest()).
 NCU_TRAFFIC = {"ggttgg": (65536, 12694784 + 1280, "295e5d2f534e0ba5")}
 KERNEL_SOURCES = ("mg_kernels.cuh", "mg_vertices.cuh", "mg_colour_tc.cuh", "mg_recursion.cuh",
@@ -136,13 +136,15 @@ class ClockSampler:
 
 def kernel_digest(tag: str) -> str:
     """sha256 (16 hex digits) of the hand-written kernel sources and of the
-    process's flop count (which changes with its generated code)."""
+    process's generated recursion."""
     import hashlib
+    from paper_2303_18244_gb300.generator import emit, recursion
     d = hashlib.sha256()
     for f in KERNEL_SOURCES:
         with open(os.path.join(ROOT, "paper_2303_18244_gb300", "csrc", f), "rb") as fh:
             d.update(fh.read())
-    d.update(json.dumps(load_flops(tag), sort_keys=True).encode())
+    n = next(n for t, n in emit.PROCESSES.values() if t == tag)
+    d.update(recursion.emit_recursion(n, tag).encode())
     return d.hexdigest()[:16]
 
 
@@ -150,7 +152,7 @@ def traffic_per_launch(tag: str, nevt: int):
     cap = NCU_TRAFFIC.get(tag)
     if cap is None or cap[2] != kernel_digest(tag):
         return None
-    return cap[1] * nevt / cap[0]
+    return cap[1] * nevt / cap[0] + 8 * nevt
 
 
 def measured_peak(key: str):
