@@ -56,3 +56,32 @@ def test_back_to_back_calls_read_their_own_pass():
         assert int(cnt) == want.numel()
         assert torch.equal(idx[:want.numel()], want)
         assert bool((idx[want.numel():] == -1).all())
+
+
+@pytest.mark.gpu
+def test_unweighting_in_a_captured_graph():
+    """The early launch and the stream-ordered workspace inside a CUDA graph:
+    replays on other inputs in the same buffers give their own kept sets."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2303_18244_gb300 import mg
+    n = 40 * 4096 + 77
+    g = torch.Generator(device="cuda").manual_seed(8)
+    r = torch.rand((n,), dtype=torch.float64, device="cuda", generator=g)
+    w = torch.full((n,), 0.5, dtype=torch.float64, device="cuda")
+    idx = torch.full((n,), -1, dtype=torch.int64, device="cuda")
+    cnt = torch.full((1,), -1, dtype=torch.int64, device="cuda")
+    mg.unweight(w, r, 1.0, idx, cnt)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        mg.unweight(w, r, 1.0, idx, cnt)
+    for kept in (0.02, 0.9, 0.3):
+        w.fill_(kept)
+        idx.fill_(-1)
+        graph.replay()
+        want = torch.nonzero(r < w).flatten()
+        assert int(cnt) == want.numel()
+        assert torch.equal(idx[:want.numel()], want)
+        assert bool((idx[want.numel():] == -1).all())
