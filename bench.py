@@ -61,7 +61,7 @@ L2_FLUSH_BYTES = 256 << 20
 # scaled to a launch by its events.  The writes are counted, 8 bytes per event:
 # the results of a capture of this size stay in L2.  Reported as null once the
 # sources differ from the captured ones (kernel_digest()).
-NCU_TRAFFIC = {"ggttgg": (65536, 12694784 + 1280, "295e5d2f534e0ba5")}
+NCU_TRAFFIC = {"ggttgg": (65536, 12694784, "59e02bd718213d0f")}
 KERNEL_SOURCES = ("mg_kernels.cuh", "mg_vertices.cuh", "mg_colour_tc.cuh", "mg_recursion.cuh",
                   "mg_recursion_kernels.cuh")
 

@@ -1,7 +1,9 @@
 // mg_kernels.cuh -- kernel templates of the matrix-element hot path.
 //
 // One event per thread, lockstep across the warp (paper Sect. 1: data
-// parallelism with lockstep processing over the events of a batch):
+// parallelism with lockstep processing over the events of a batch).  gg -> t t~
+// + gluons runs the recursion of mg_recursion_kernels.cuh instead, except for
+// the helicity and colour choice of the FP32 modes:
 //   A1  the CTA's momenta tile (NT events x NPAR x 4 doubles, contiguous) is
 //       copied global -> shared by the TMA engine (cp.async.bulk, completion
 //       on an mbarrier with a bounded wait);
@@ -12,9 +14,10 @@
 //   A3-A4  per good helicity (uniform across the CTA): wavefunctions,
 //       off-shell currents and amplitudes diagram by diagram, accumulated
 //       into the colour flows (generated straight-line code);
-//   A5  colour quadratic form J^dagger C J (FP64 FMA in the FP64 path; on
-//       the tensor cores in the mixed path, see mg_colour_tc.cuh);
-//   A6  helicity sum in FP64, normalised by 1/(IDEN * CDEN), one store.
+//   A5  colour quadratic form J^dagger C J (FMAs in the precision of the
+//       flows; FP32 in the paper's mixed mode);
+//   A6  helicity sum in FP64 (FP32 in the all-float mode), normalised by
+//       1/(IDEN * CDEN), one store.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -194,8 +197,9 @@ __device__ __forceinline__ unsigned good_mask(const int* __restrict__ hels, int 
   return __reduce_or_sync(0xffffffffu, lane < nhel ? 1u << __ldg(hels + lane) : 0u);
 }
 
-// |M|^2 by one thread per event that runs every helicity in registers
-// (P::thread_sum): the small processes, whose currents fit.  Each current is
+// |M|^2 by one thread per event that runs every helicity (P::thread_sum): the
+// small processes, whose currents fit in its registers (FP32: 80 to 104 bytes
+// are spilled; FP64: 0.5 KB of gg -> t t~, 2.6 KB of u u~ -> t t~ g).  Each current is
 // computed once per helicity combination of its own legs: a third of the
 // instructions of sigma_kernel, which evaluates every helicity by itself.
 // CTAS: CTAs per SM the registers are sized for.  Measured (us): g g -> t t~,

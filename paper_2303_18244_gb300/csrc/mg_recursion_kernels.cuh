@@ -23,9 +23,9 @@ struct RecShape {
   // helicity: five gluons (registers), and four in FP64, where the flows of one
   // helicity leave room for 12 warps (six events, the late vectors over others)
   // instead of 4, and 12 keep the FP64 pipe busier: 32749 events 11.3 -> 9.97 ms
-  // (8 / 10 warps 10.2 / 10.5).  In FP32 the antitop spins share the loads of
-  // the rows: 4.66 ms for 524288 events against 5.8 / 5.5 / 5.4 ms with a thread
-  // per helicity and 24 / 20 / 16 warps.  Three gluons, FP64, 65536 events: 2.88
+  // (8 / 10 warps 10.2 / 10.5), though 0.3 KB a thread are spilled.  In FP32 the
+  // antitop spins share the loads of the rows: 4.76 ms for 524288 events against
+  // 5.8 / 5.5 / 5.4 ms with a thread per helicity and 24 / 20 / 16 warps.  Three gluons, FP64, 65536 events: 2.88
   // against 2.92 .. 3.6 ms.
   static constexpr int T = P::N == 5 || (P::N == 4 && !f32) ? P::NHEL : 1 << (P::N + 1);
   // warps of a CTA, a multiple of the four schedulers.  Measured, 524288 events

@@ -168,8 +168,11 @@ __global__ void __launch_bounds__(SCAN_T) tile_scan_kernel(long long* __restrict
 // Last pass: a warp per tile, WRITE_TILES tiles per block.  The kept events
 // before the block's first tile: SCANNED, from the scan; otherwise the block
 // adds up the counts of all earlier tiles (ntiles^2 / 4 bytes of L2 reads over
-// all blocks, 67 MB at SUM_TILES tiles, about what the scan of one block and
-// its launch cost there).  33.6 M events, 2.7 % kept: count 78 + scan 8 + a
+// all blocks, 67 MB at SUM_TILES tiles).  A call with the sum / with the scan,
+// us: 512 tiles 35.0 / 45.0, 4096 69.9 / 76.8, 8192 113 / 119, 16384 193 / 201,
+// 24576 273 / 286, 32768 357 / 365, 65536 708 / 705; the reads grow with the
+// square of the tiles, and the line stays a factor of two below the crossing.
+// 33.6 M events, 2.7 % kept: count 78 + scan 8 + a
 // block per tile 22 us before; count 78 + write 9 us now, 111.8 -> 92.4 us a
 // call; 8 / 16 / 32 tiles per block 91.9 / 92.4 / 93.2 us; without the early
 // launch 96.4 us.

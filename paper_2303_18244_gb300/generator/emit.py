@@ -1252,16 +1252,17 @@ def _prepare_in_D(src: str) -> str:
     return "\n".join(lines[:i1 + 1] + body + lines[i2:])
 
 
-# threads per CTA: FP64 path / mixed path (shared-memory slab sizes differ)
+# threads per CTA of the per-helicity program: FP64 path (None: the recursion
+# runs it) / mixed path (shared-memory slab sizes differ)
 THREADS = {
     "eemumu": (128, 128),
     "uutt": (128, 128),
     "uuttg": (128, 128),
     "uuttgg": (64, 128),
-    "ggtt": (128, 128),
-    "ggttg": (128, 128),
-    "ggttgg": (64, 128),
-    "ggttggg": (64, 64),
+    "ggtt": (None, 128),
+    "ggttg": (None, 128),
+    "ggttgg": (None, 128),
+    "ggttggg": (None, 64),
 }
 
 
